@@ -412,8 +412,9 @@ int64_t bsvd_panel_launches(const bsvd_ctx *ctx);
  *   * Schedule (Section 3, Figure 2): the blocks of the last bsvd_partition
  *     grid are visited in steps of blocks that share no block row and no
  *     block column: step s holds blocks ((j + s) mod p, j), j < q, when
- *     p >= q, else (i, (i + s) mod q), i < p. The blocks of a step run at
- *     once, one warp each.
+ *     p >= q, else (i, (i + s) mod q), i < p. The results are those
+ *     of the ratings one after another in this order; ratings that share no
+ *     user and no item with an unfinished earlier one run at the same time.
  *   * Within a block (Algorithm 2): its ratings row by row, then column by
  *     column. For each rating, with err = x - bu - bi - p . q:
  *       bu += a_ubias (err - b_ubias bu),  bi += a_ibias (err - b_ibias bi),
@@ -428,14 +429,12 @@ int64_t bsvd_panel_launches(const bsvd_ctx *ctx);
  *   * BSVD_SGD_FP64 (the default): float64 with one rounding per operation
  *     (no fused multiply-add) and the dot product summed over f = 0 .. k-1
  *     in order, so results equal a sequential float64 implementation bit
- *     for bit. A block's walk is a chain of dependent float64 operations.
+ *     for bit.
  *   * BSVD_SGD_FP32: the same operations in the same order in float32 (no
  *     fused multiply-add), on float32 copies of P0, Q0 (rounded to nearest)
- *     and rates rounded to float32; each block stages its users' and items'
- *     parameters in shared memory when they fit (else it works in global
- *     memory). Results equal a sequential float32 implementation bit for
- *     bit. The RMSE, bsvd_sgd_predict and bsvd_sgd_get see the float32
- *     values widened to float64.
+ *     and rates rounded to float32. Results equal a sequential float32
+ *     implementation bit for bit. The RMSE, bsvd_sgd_predict and
+ *     bsvd_sgd_get see the float32 values widened to float64.
  */
 typedef enum {
     BSVD_SGD_FP64 = 0,
@@ -481,7 +480,7 @@ bsvd_status bsvd_sgd_prepare(bsvd_ctx *ctx, int64_t nnz, const int32_t *u,
  * before the first epoch, then after each epoch run. *steps_run (may be
  * NULL): epochs run.
  * Errors: BSVD_ESTATE (no bsvd_sgd_prepare), BSVD_EINVAL (parameters),
- * BSVD_ENOMEM, BSVD_ECUDA.
+ * BSVD_ENOMEM, BSVD_ECUDA, BSVD_ETIMEOUT (a device-side wait gave up).
  */
 bsvd_status bsvd_sgd_train(bsvd_ctx *ctx, const bsvd_sgd_params *prm,
                            const double *P0, const double *Q0, double *rmse,

@@ -151,15 +151,16 @@ struct bsvd_ctx {
   std::vector<unsigned char> fsig;
   DevBuf d_state0;
 
-  // blocked SGD (Algorithms 1-2): ratings in epoch order, block ranges,
-  // schedule, model
+  // blocked SGD (Algorithms 1-2): ratings in epoch order, tasks, the
+  // versions they wait for, and the model
   bool sgd_ready = false, sgd_trained = false;
   int64_t sgd_nnz = 0;
   int32_t sgd_k = 0;
-  DevBuf d_sgd_cnt, d_sgd_off, d_sgd_key, d_sgd_src, d_sgd_u, d_sgd_i,
-      d_sgd_x, d_sgd_r, d_sgd_c, d_sgd_range, d_sgd_blocks, d_sgd_P,
-      d_sgd_Q, d_sgd_bu, d_sgd_bi, d_sgd_sum, d_sgd_P32, d_sgd_Q32;
-  std::vector<int32_t> sgd_step_off;   // steps: blocks [off[s], off[s+1])
+  int32_t sgd_own_items = 1;
+  DevBuf d_sgd_key[2], d_sgd_src[2], d_sgd_hist, d_sgd_start, d_sgd_first,
+      d_sgd_ntasks, d_sgd_u, d_sgd_i, d_sgd_x, d_sgd_ov, d_sgd_wv, d_sgd_P,
+      d_sgd_Q, d_sgd_bu, d_sgd_bi, d_sgd_sum, d_sgd_prow, d_sgd_qrow,
+      d_sgd_ctl;
   bool any_capped = false;
 
   // staging of host arguments and results
@@ -564,11 +565,13 @@ void bsvd_destroy(bsvd_ctx *c) {
                     &c->d_shift, &c->d_delta, &c->d_maps, &c->d_flag,
                     &c->d_wmaps, &c->d_ptiles, &c->d_gmaps, &c->d_xmaps, &c->d_XB, &c->d_ZB,
                     &c->d_pjtiles, &c->d_pwmaps, &c->d_state0,
-                    &c->d_sgd_cnt, &c->d_sgd_off, &c->d_sgd_key,
-                    &c->d_sgd_src, &c->d_sgd_u, &c->d_sgd_i, &c->d_sgd_x,
-                    &c->d_sgd_range, &c->d_sgd_blocks, &c->d_sgd_P,
-                    &c->d_sgd_Q, &c->d_sgd_bu, &c->d_sgd_bi, &c->d_sgd_sum,
-                    &c->d_sgd_r, &c->d_sgd_c, &c->d_sgd_P32, &c->d_sgd_Q32,
+                    &c->d_sgd_key[0], &c->d_sgd_key[1], &c->d_sgd_src[0],
+                    &c->d_sgd_src[1], &c->d_sgd_hist, &c->d_sgd_start,
+                    &c->d_sgd_first, &c->d_sgd_ntasks, &c->d_sgd_u,
+                    &c->d_sgd_i, &c->d_sgd_x, &c->d_sgd_ov, &c->d_sgd_wv,
+                    &c->d_sgd_P, &c->d_sgd_Q, &c->d_sgd_bu, &c->d_sgd_bi,
+                    &c->d_sgd_sum, &c->d_sgd_prow, &c->d_sgd_qrow,
+                    &c->d_sgd_ctl,
                     &c->d_qcnt, &c->d_qkeys, &c->d_qcum, &c->d_qperm,
                     &c->d_qperm2,
                     &c->d_qbounds, &c->d_pbmaps, &c->d_fbmaps, &c->d_FB,
@@ -2010,60 +2013,54 @@ bsvd_status bsvd_sgd_prepare(bsvd_ctx *c, int64_t nnz, const int32_t *u,
   c->sgd_ready = false;
   c->sgd_trained = false;
   const GridDesc g = c->grid();
-  const int32_t nb = c->nblocks;
-  const int64_t nbuckets = (int64_t)(c->diag ? c->p : c->q) * c->m;
   const void *du = u, *di = i, *dx = x;
   CK(device_view(c, u, sizeof(int32_t) * nnz, c->s_a, &du), "sgd_prepare");
   CK(device_view(c, i, sizeof(int32_t) * nnz, c->s_b, &di), "sgd_prepare");
   CK(device_view(c, x, sizeof(float) * nnz, c->s_c, &dx), "sgd_prepare");
   const size_t n1 = (size_t)std::max<int64_t>(nnz, 1);
-  // bucket counts, then (from the sort on) the list of large buckets
-  CK(c->d_sgd_cnt.ensure(sizeof(unsigned long long) * (nbuckets + 1)),
-     "sgd_prepare");
-  CK(c->d_sgd_off.ensure(sizeof(int64_t) * (nbuckets + 1)), "sgd_prepare");
-  CK(c->d_sgd_key.ensure(sizeof(int64_t) * n1), "sgd_prepare");
-  CK(c->d_sgd_src.ensure(sizeof(int64_t) * n1), "sgd_prepare");
+  const size_t ib = sgd_index_bytes(nnz);
+  SgdOrder o;
+  o.own_items = c->n <= c->m ? 1 : 0;
+  o.max_rows = o.max_cols = 1;
+  for (int32_t j = 0; j < c->p; ++j)
+    o.max_rows = std::max(o.max_rows, c->rb[j + 1] - c->rb[j]);
+  for (int32_t j = 0; j < c->q; ++j)
+    o.max_cols = std::max(o.max_cols, c->cb[j + 1] - c->cb[j]);
+  for (int h = 0; h < 2; ++h) {
+    CK(c->d_sgd_key[h].ensure(sizeof(int64_t) * n1), "sgd_prepare");
+    CK(c->d_sgd_src[h].ensure(ib * n1), "sgd_prepare");
+    o.key[h] = c->d_sgd_key[h].p;
+    o.val[h] = c->d_sgd_src[h].p;
+  }
+  CK(c->d_sgd_hist.ensure(sgd_hist_bytes(nnz)), "sgd_prepare");
+  CK(c->d_sgd_start.ensure(ib * (size_t)std::max(c->m, c->n)), "sgd_prepare");
+  // an owner has at most one task in each block of its block row or column
+  const int64_t tmax = std::min<int64_t>(
+      nnz, c->diag ? (o.own_items ? c->n : c->m)
+                   : (o.own_items ? (int64_t)c->p * c->n
+                                  : (int64_t)c->q * c->m));
+  CK(c->d_sgd_first.ensure(ib * (size_t)(tmax + 1)), "sgd_prepare");
+  CK(c->d_sgd_ntasks.ensure(sizeof(int64_t)), "sgd_prepare");
   CK(c->d_sgd_u.ensure(sizeof(int32_t) * n1), "sgd_prepare");
   CK(c->d_sgd_i.ensure(sizeof(int32_t) * n1), "sgd_prepare");
   CK(c->d_sgd_x.ensure(sizeof(float) * n1), "sgd_prepare");
-  CK(c->d_sgd_r.ensure(sizeof(int32_t) * n1), "sgd_prepare");
-  CK(c->d_sgd_c.ensure(sizeof(int32_t) * n1), "sgd_prepare");
-  CK(c->d_sgd_range.ensure(sizeof(int64_t) * 2 * nb), "sgd_prepare");
-  CK(launch_sgd_order(g, nb, nnz, (const int32_t *)du, (const int32_t *)di,
-                      (const float *)dx, c->d_sgd_cnt.as<unsigned long long>(),
-                      c->d_sgd_off.as<int64_t>(), c->d_sgd_key.as<int64_t>(),
-                      c->d_sgd_src.as<int64_t>(), c->d_sgd_u.as<int32_t>(),
-                      c->d_sgd_i.as<int32_t>(), c->d_sgd_x.as<float>(),
-                      c->d_sgd_r.as<int32_t>(), c->d_sgd_c.as<int32_t>(),
-                      c->d_sgd_range.as<int64_t>(), c->d_err.as<int32_t>(),
+  CK(c->d_sgd_ov.ensure(sizeof(unsigned) * n1), "sgd_prepare");
+  CK(c->d_sgd_wv.ensure(sizeof(unsigned) * n1), "sgd_prepare");
+  o.hist = c->d_sgd_hist.p;
+  o.start = c->d_sgd_start.p;
+  o.task_first = c->d_sgd_first.p;
+  o.ntasks = c->d_sgd_ntasks.as<int64_t>();
+  o.su = c->d_sgd_u.as<int32_t>();
+  o.si = c->d_sgd_i.as<int32_t>();
+  o.sx = c->d_sgd_x.as<float>();
+  o.other_ver = c->d_sgd_ov.as<unsigned>();
+  o.own_ver = c->d_sgd_wv.as<unsigned>();
+  CK(launch_sgd_order(g, o, nnz, (const int32_t *)du, (const int32_t *)di,
+                      (const float *)dx, &c->launches, c->d_err.as<int32_t>(),
                       c->st), "sgd_prepare");
-  c->launches += nnz > 0 ? 7 : 2;
   bsvd_status s = read_errors(c, "sgd_prepare");
   if (s != BSVD_OK) return s;
-  // the diagonal schedule (Figure 2): blocks sharing no block row or column
-  std::vector<int32_t> blocks;
-  c->sgd_step_off.assign(1, 0);
-  if (c->diag) {
-    for (int32_t b = 0; b < nb; ++b) blocks.push_back(b);
-    c->sgd_step_off.push_back(nb);
-  } else if (c->p >= c->q) {
-    for (int32_t st = 0; st < c->p; ++st) {
-      for (int32_t j = 0; j < c->q; ++j)
-        blocks.push_back(((j + st) % c->p) * c->q + j);
-      c->sgd_step_off.push_back((int32_t)blocks.size());
-    }
-  } else {
-    for (int32_t st = 0; st < c->q; ++st) {
-      for (int32_t r = 0; r < c->p; ++r)
-        blocks.push_back(r * c->q + (r + st) % c->q);
-      c->sgd_step_off.push_back((int32_t)blocks.size());
-    }
-  }
-  CK(c->d_sgd_blocks.ensure(sizeof(int32_t) * blocks.size()), "sgd_prepare");
-  CK(cudaMemcpyAsync(c->d_sgd_blocks.p, blocks.data(),
-                     sizeof(int32_t) * blocks.size(), cudaMemcpyHostToDevice,
-                     c->st), "sgd_prepare");
-  CK(cudaStreamSynchronize(c->st), "sgd_prepare");
+  c->sgd_own_items = o.own_items;
   c->sgd_nnz = nnz;
   c->sgd_ready = true;
   return BSVD_OK;
@@ -2119,76 +2116,48 @@ bsvd_status bsvd_sgd_train(bsvd_ctx *c, const bsvd_sgd_params *prm,
   const SgdRates r{prm->a_user, prm->b_user, prm->a_item, prm->b_item,
                    prm->a_ubias, prm->b_ubias, prm->a_ibias, prm->b_ibias};
   const bool f32 = prm->precision == BSVD_SGD_FP32;
-  const SgdRates32 r32{(float)prm->a_user,  (float)prm->b_user,
-                       (float)prm->a_item,  (float)prm->b_item,
-                       (float)prm->a_ubias, (float)prm->b_ubias,
-                       (float)prm->a_ibias, (float)prm->b_ibias};
-  size_t stage = 0;
-  if (f32) {
-    // float32 rows of k + 1 (factors, bias); the float64 arrays then hold
-    // their widened values, which the RMSE, predict and get read
-    CK(c->d_sgd_P32.ensure(sizeof(float) * (size_t)std::max<int64_t>(
-                               c->m * (k + 1), 1)), "sgd_train");
-    CK(c->d_sgd_Q32.ensure(sizeof(float) * (size_t)std::max<int64_t>(
-                               c->n * (k + 1), 1)), "sgd_train");
-    CK(launch_sgd_narrow(c->m, c->n, k, c->d_sgd_P.as<double>(),
-                         c->d_sgd_Q.as<double>(), c->d_sgd_bu.as<double>(),
-                         c->d_sgd_bi.as<double>(), c->d_sgd_P32.as<float>(),
-                         c->d_sgd_Q32.as<float>(), c->st), "sgd_train");
-    CK(launch_sgd_widen(c->m, c->n, k, c->d_sgd_P32.as<float>(),
-                        c->d_sgd_Q32.as<float>(), c->d_sgd_P.as<double>(),
-                        c->d_sgd_Q.as<double>(), c->d_sgd_bu.as<double>(),
-                        c->d_sgd_bi.as<double>(), c->st), "sgd_train");
-    c->launches += 2;
-    // stage the blocks in shared memory when the largest one fits
-    int dev = 0, optin = 0;
-    CK(cudaGetDevice(&dev), "sgd_train");
-    CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin,
-                              dev), "sgd_train");
-    for (int32_t b = 0; b < c->nblocks; ++b) {
-      const int32_t bi = c->diag ? b : b / c->q, bj = c->diag ? b : b % c->q;
-      stage = std::max(stage, sgd_stage_bytes(c->rb[bi + 1] - c->rb[bi],
-                                              c->cb[bj + 1] - c->cb[bj], k));
-    }
-    if (stage > (size_t)optin) stage = 0;
-  }
-  const GridDesc g = c->grid();
+  // the parameters as the epochs keep them; in the float32 form the float64
+  // arrays then hold their widened values, which the RMSE, predict and get
+  // read
+  CK(c->d_sgd_prow.ensure(sgd_row_bytes(k, f32) * (size_t)std::max<int64_t>(
+                              c->m, 1)), "sgd_train");
+  CK(c->d_sgd_qrow.ensure(sgd_row_bytes(k, f32) * (size_t)std::max<int64_t>(
+                              c->n, 1)), "sgd_train");
+  CK(c->d_sgd_ctl.ensure(3 * sizeof(unsigned long long)), "sgd_train");
+  auto rows = [&](int pack) {
+    ++c->launches;
+    return launch_sgd_rows(pack, f32, c->m, c->n, k, c->d_sgd_P.as<double>(),
+                           c->d_sgd_Q.as<double>(), c->d_sgd_bu.as<double>(),
+                           c->d_sgd_bi.as<double>(), c->d_sgd_prow.p,
+                           c->d_sgd_qrow.p, c->d_sgd_ctl.as<unsigned long long>(), c->st);
+  };
+  CK(rows(1), "sgd_train");
+  if (f32) CK(rows(0), "sgd_train");
+  SgdEpoch ep;
+  ep.task_first = c->d_sgd_first.p;
+  ep.ntasks = c->d_sgd_ntasks.as<int64_t>();
+  const bool oi = c->sgd_own_items != 0;
+  ep.own = oi ? c->d_sgd_i.as<int32_t>() : c->d_sgd_u.as<int32_t>();
+  ep.other = oi ? c->d_sgd_u.as<int32_t>() : c->d_sgd_i.as<int32_t>();
+  ep.x = c->d_sgd_x.as<float>();
+  ep.other_ver = c->d_sgd_ov.as<unsigned>();
+  ep.own_ver = c->d_sgd_wv.as<unsigned>();
+  ep.own_rows = (oi ? c->d_sgd_qrow : c->d_sgd_prow).as<unsigned long long>();
+  ep.other_rows = (oi ? c->d_sgd_prow : c->d_sgd_qrow).as<unsigned long long>();
+  ep.r = r;
+  ep.own_items = c->sgd_own_items;
+  ep.k = k;
+  ep.ctl = c->d_sgd_ctl.as<unsigned long long>();
+  ep.err = c->d_err.as<int32_t>();
   double prev = 0.0;
   bsvd_status s = sgd_rmse(c, &prev);
   if (s != BSVD_OK) return s;
   if (rmse) rmse[0] = prev;
   int32_t ran = 0;
   for (int32_t step = 0; step < prm->max_steps; ++step) {
-    for (size_t t = 0; t + 1 < c->sgd_step_off.size(); ++t) {
-      const int32_t a = c->sgd_step_off[t], b = c->sgd_step_off[t + 1];
-      if (f32)
-        CK(launch_sgd_step_f32(g, b - a, c->d_sgd_blocks.as<int32_t>() + a,
-                               c->d_sgd_range.as<int64_t>(),
-                               c->d_sgd_r.as<int32_t>(),
-                               c->d_sgd_c.as<int32_t>(),
-                               c->d_sgd_u.as<int32_t>(),
-                               c->d_sgd_i.as<int32_t>(),
-                               c->d_sgd_x.as<float>(), c->sgd_nnz, k,
-                               c->d_sgd_P32.as<float>(),
-                               c->d_sgd_Q32.as<float>(), r32, stage,
-                               c->d_err.as<int32_t>(), c->st), "sgd_train");
-      else
-        CK(launch_sgd_step(b - a, c->d_sgd_blocks.as<int32_t>() + a,
-                           c->d_sgd_range.as<int64_t>(),
-                           c->d_sgd_u.as<int32_t>(), c->d_sgd_i.as<int32_t>(),
-                           c->d_sgd_x.as<float>(), c->sgd_nnz, k,
-                           c->d_sgd_P.as<double>(), c->d_sgd_Q.as<double>(),
-                           c->d_sgd_bu.as<double>(), c->d_sgd_bi.as<double>(),
-                           r, c->d_err.as<int32_t>(), c->st), "sgd_train");
-      c->launches += 1;
-    }
-    if (f32) {
-      CK(launch_sgd_widen(c->m, c->n, k, c->d_sgd_P32.as<float>(),
-                          c->d_sgd_Q32.as<float>(), c->d_sgd_P.as<double>(),
-                          c->d_sgd_Q.as<double>(), c->d_sgd_bu.as<double>(),
-                          c->d_sgd_bi.as<double>(), c->st), "sgd_train");
-      c->launches += 1;
-    }
+    CK(launch_sgd_epoch(ep, c->sgd_nnz, f32, c->nsm, c->st), "sgd_train");
+    c->launches += c->sgd_nnz > 0;
+    CK(rows(0), "sgd_train");
     ++ran;
     double cur = 0.0;
     s = sgd_rmse(c, &cur);
