@@ -1917,11 +1917,6 @@ bsvd_status bsvd_reconstruct(bsvd_ctx *c, int32_t b, int32_t add_mean,
                 "context (bsvd_set_owned)", b);
   const size_t cells = (size_t)bm.mb * bm.nb;
   if (cells == 0) return BSVD_OK;
-  float mu = 0.f;
-  if (add_mean)
-    CK(cudaMemcpyAsync(&mu, c->d_mu.as<float>() + b, sizeof mu,
-                       cudaMemcpyDeviceToHost, c->st), "reconstruct");
-  CK(cudaStreamSynchronize(c->st), "reconstruct");
   const bool dev_out = is_device_ptr(out);
   float *dst = out;
   if (!dev_out) {
@@ -1929,7 +1924,8 @@ bsvd_status bsvd_reconstruct(bsvd_ctx *c, int32_t b, int32_t add_mean,
     dst = c->s_out.as<float>();
   }
   CK(launch_reconstruct(c->d_meta.as<BlockMeta>(), bm, b, c->d_Fs.as<float>(),
-                        c->d_FL.as<float>(), c->kp, mu, dst,
+                        c->d_FL.as<float>(), c->kp,
+                        add_mean ? c->d_mu.as<float>() : nullptr, dst,
                         c->d_err.as<int32_t>(), c->st),
      "reconstruct");
   c->launches += 1;
