@@ -172,8 +172,9 @@ struct GridDesc {
 };
 
 // Largest j with bounds[j] <= v, for bounds[0] = 0 <= v < bounds[count].
-__device__ __forceinline__ int32_t upper_index(const int64_t *bounds,
-                                               int32_t count, int64_t v) {
+template <typename I>
+__device__ __forceinline__ int32_t upper_index(const I *bounds, int32_t count,
+                                               I v) {
   int32_t lo = 0, hi = count;       // invariant: bounds[lo] <= v < bounds[hi]
   while (hi - lo > 1) {
     int32_t mid = (lo + hi) >> 1;
@@ -183,17 +184,19 @@ __device__ __forceinline__ int32_t upper_index(const int64_t *bounds,
 }
 
 // Block id and local (row, col) of a rating; false if an id is out of range.
+// Positions and block sizes are below 2^31 (m and n are), so the divisions
+// are 32-bit ones.
 __device__ __forceinline__ bool locate(const GridDesc &g, int32_t u,
                                        int32_t i, int32_t *blk, int32_t *r,
                                        int32_t *c) {
   if (u < 0 || (int64_t)u >= g.m || i < 0 || (int64_t)i >= g.n) return false;
-  int64_t ru = g.row_perm ? (int64_t)g.row_perm[u] : (int64_t)u;
-  int64_t ci = g.col_perm ? (int64_t)g.col_perm[i] : (int64_t)i;
+  const int32_t ru = g.row_perm ? g.row_perm[u] : u;
+  const int32_t ci = g.col_perm ? g.col_perm[i] : i;
   int32_t bi, bj;
-  if (g.equal_rows) bi = (int32_t)(ru / g.br);
-  else bi = upper_index(g.row_bounds, g.p, ru);
-  if (g.equal_cols) bj = (int32_t)(ci / g.bc);
-  else bj = upper_index(g.col_bounds, g.q, ci);
+  if (g.equal_rows) bi = (int32_t)((uint32_t)ru / (uint32_t)g.br);
+  else bi = upper_index(g.row_bounds, g.p, (int64_t)ru);
+  if (g.equal_cols) bj = (int32_t)((uint32_t)ci / (uint32_t)g.bc);
+  else bj = upper_index(g.col_bounds, g.q, (int64_t)ci);
   if (g.diag) {
     if (bi != bj) return false;     // off the block diagonal
     *blk = bi;
