@@ -93,6 +93,18 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
 }
 constexpr int KC = 32;       // k-chunk of the panel GEMM
 
+// a / b, rounded to nearest, given inv = 1 / b rounded to nearest (Markstein's
+// theorem, "Computation of elementary functions on the IBM RISC System/6000
+// processor", 1990: with the remainder a - b q of a quotient q within one unit
+// in the last place, exact in a fused multiply-add, q + r inv rounds to the
+// nearest). The first correction makes q that close. For operands whose
+// quotient and remainder do not underflow.
+__device__ __forceinline__ float quotient(float a, float b, float inv) {
+  float q = a * inv;
+  q = fmaf(fmaf(-b, q, a), inv, q);
+  return fmaf(fmaf(-b, q, a), inv, q);
+}
+
 __device__ __forceinline__ float hash_uniform(uint64_t seed, uint64_t a,
                                               uint64_t b) {
   // splitmix64 of (seed, a, b) -> uniform in [-1, 1)
@@ -395,53 +407,87 @@ __device__ __forceinline__ void build_pairs(int ne, unsigned short *tab) {
 // orthonormal U, and for a PSD A the columns of V are its eigenvectors and
 // the column norms |A v_j| its eigenvalues.
 // Round-robin ordering gives np disjoint pairs per round. Each half-warp
-// takes one pair (a warp two: pairs 2w + h, 2 (w + nwarps) + h, ...), lane
-// l of the half holding rows l, l + 16, ... of the two columns. The three
-// dot products are xor-butterfly sums over the half-warp: each step adds
-// the same two operands in every lane, so the 16 lanes hold bitwise equal
-// sums and apply the same rotation. The loop is issue-bound (one warp per
-// pair took about 1600 cycles a round at b = 64: 32 warps' shuffles and
-// address arithmetic), so two pairs per warp halve the instructions per
-// round. One block-wide barrier per round.
+// takes one pair (warp w the pairs 2 w and 2 w + 1; the other warps of the
+// CTA wait for the end), lane l of the half holding rows l, l + 16, ... of
+// the two columns. A column is stored in that order (row_at), so a lane's
+// rows are one load of up to 16 bytes. The three dot products are
+// xor-butterfly sums over the half-warp: each step adds the same two
+// operands in every lane, so the 16 lanes hold bitwise equal sums and apply
+// the same rotation.
+// A round is a chain: loads, dot products, four butterfly steps, the angle,
+// the update, a barrier. So what helps is what shortens the chain: the next
+// round's pair is looked up before the barrier, the columns of V are loaded
+// with those of A, only the working warps meet at the barrier (28 cycles for
+// eight warps, 77 for 32), and the last round's barrier carries whether any
+// pair of the sweep rotated. At b = 32 a round takes 485 cycles (750 with
+// scalar loads, a look-up after the barrier, and all 32 warps at it), at b = 64
+// 760 (1,280).
 template <int B>
-__device__ int onesided_jacobi(float (*Ac)[B + 1], float (*Vc)[B + 1], int n,
+__device__ __forceinline__ int row_at(int r) {
+  return (r & 15) * (B / 16) + (r >> 4);
+}
+
+// Barrier of the first `threads` threads of the CTA (whole warps), and the
+// same returning whether `p` holds for any of them.
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ bool bar_or(int id, int threads, bool p) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred a, b;\n\tsetp.ne.s32 a, %3, 0;\n\t"
+      "bar.red.or.pred b, %1, %2, a;\n\tselp.s32 %0, 1, 0, b;\n\t}"
+      : "=r"(r)
+      : "r"(id), "r"(threads), "r"((int)p)
+      : "memory");
+  return r != 0;
+}
+
+// Called by the first ceil(np / 2) warps (the CTA has at least B / 4); rows
+// n .. B - 1 of every column are zero. Returns the sweeps that rotated.
+template <int B, int P>
+__device__ int onesided_jacobi(float (*Ac)[P], float (*Vc)[P], int n,
                                int max_sweeps, const unsigned short *pairs,
-                               int *flag, float tol) {
-  constexpr int RPL = (B + 15) / 16;        // rows per lane
+                               float tol) {
+  constexpr int RPL = B / 16;               // rows per lane
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int hl = lane & 15, half = lane >> 4;
-  const int nwarps = blockDim.x >> 5;
   const int ne = n + (n & 1), np = ne / 2;
+  const int threads = 32 * ((np + 1) / 2);
+  const int i = 2 * warp + half;            // this half-warp's pair
+  const bool has = i < np;
+  const unsigned short *mine = pairs + (has ? i : 0);
+  const float tol2 = tol * tol;
   int sweep = 0;
+  unsigned pq = mine[0];
   for (; sweep < max_sweeps; ++sweep) {
-    if (threadIdx.x == 0) *flag = 0;
-    __syncthreads();
+    bool rotated = false;
     for (int round = 0; round < ne - 1; ++round) {
-      const unsigned short *pr = pairs + round * np;
-      // warp-uniform trip count: both halves run the shuffles
-      for (int w2 = warp; 2 * w2 < np; w2 += nwarps) {
-        const int i = 2 * w2 + half;
-        const bool has = i < np;
-        const int p = has ? (pr[i] & 255) : 0, q = has ? (pr[i] >> 8) : 0;
-        const bool valid = has && p < n && q < n;
-        float a[RPL], b[RPL];
-        float al = 0.f, be = 0.f, ga = 0.f;
+      const int p = pq & 255, q = pq >> 8;
+      const bool valid = has && p < n && q < n;
+      float *ap = &Ac[valid ? p : 0][RPL * hl], *aq = &Ac[valid ? q : 0][RPL * hl];
+      float *vp = &Vc[valid ? p : 0][RPL * hl], *vq = &Vc[valid ? q : 0][RPL * hl];
+      float a[RPL], b[RPL], va[RPL], vb[RPL];
+      ld_vec(ap, a);
+      ld_vec(aq, b);
+      ld_vec(vp, va);
+      ld_vec(vq, vb);
+      const int next = round + 1 < ne - 1 ? round + 1 : 0;
+      pq = mine[next * np];
+      float al = 0.f, be = 0.f, ga = 0.f;
 #pragma unroll
-        for (int h = 0; h < RPL; ++h) {
-          const int r = hl + 16 * h;
-          a[h] = (valid && r < n) ? Ac[p][r] : 0.f;
-          b[h] = (valid && r < n) ? Ac[q][r] : 0.f;
-          al = fmaf(a[h], a[h], al);
-          be = fmaf(b[h], b[h], be);
-          ga = fmaf(a[h], b[h], ga);
-        }
+      for (int h = 0; h < RPL; ++h) {
+        al = fmaf(a[h], a[h], al);
+        be = fmaf(b[h], b[h], be);
+        ga = fmaf(a[h], b[h], ga);
+      }
 #pragma unroll
-        for (int o = 8; o > 0; o >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, o);
-          be += __shfl_xor_sync(0xffffffffu, be, o);
-          ga += __shfl_xor_sync(0xffffffffu, ga, o);
-        }
-        if (!valid || !(ga * ga > (tol * tol) * (al * be))) continue;
+      for (int o = 8; o > 0; o >>= 1) {
+        al += __shfl_xor_sync(0xffffffffu, al, o);
+        be += __shfl_xor_sync(0xffffffffu, be, o);
+        ga += __shfl_xor_sync(0xffffffffu, ga, o);
+      }
+      if (valid && ga * ga > tol2 * (al * be)) {
         // The angle only has to be close to the optimal one (any rotation
         // near it still converges), so t uses the hardware's approximate
         // reciprocal and square root; what must be accurate is c^2 + s^2 = 1,
@@ -455,44 +501,78 @@ __device__ int onesided_jacobi(float (*Ac)[B + 1], float (*Vc)[B + 1], int n,
         float c = rsqrt_approx(x);
         c = c * fmaf(-0.5f * x, c * c, 1.5f);
         const float s = t * c;
-        if (s == 0.f) continue;
-        if (hl == 0) *flag = 1;
+        if (s != 0.f) {
+          rotated = true;
+          float na[RPL], nb[RPL], nva[RPL], nvb[RPL];
 #pragma unroll
-        for (int h = 0; h < RPL; ++h) {
-          const int r = hl + 16 * h;
-          if (r < n) {
-            Ac[p][r] = c * a[h] - s * b[h];
-            Ac[q][r] = s * a[h] + c * b[h];
-            const float va = Vc[p][r], vb = Vc[q][r];
-            Vc[p][r] = c * va - s * vb;
-            Vc[q][r] = s * va + c * vb;
+          for (int h = 0; h < RPL; ++h) {
+            na[h] = c * a[h] - s * b[h];
+            nb[h] = s * a[h] + c * b[h];
+            nva[h] = c * va[h] - s * vb[h];
+            nvb[h] = s * va[h] + c * vb[h];
           }
+          st_vec(ap, na);
+          st_vec(aq, nb);
+          st_vec(vp, nva);
+          st_vec(vq, nvb);
         }
       }
-      __syncthreads();
+      if (next) bar_sync(1, threads);
     }
-    const int any = *flag;
-    __syncthreads();
-    if (!any) break;
+    if (!bar_or(1, threads, rotated)) break;
   }
   return sweep;
 }
 
 template <int B>
 struct RRSmem {
-  float S[B][B + 1];      // S_n, then its Cholesky factor L (lower)
-  float Li[B][B + 1];     // L^-1 (lower)
-  float H[B][B + 1];
-  float T1[B][B + 1];
-  float A[B][B + 1];
-  float V[B][B + 1];
+  static constexpr int P = B + 4;           // 16-byte rows
+  float S[B][B + 1];      // S_n, then its Cholesky work, then H'
+  float Li[B][P];         // work of L^-1, then H T1, then V^T
+  float H[B][P];          // H^T, then T1^T
+  float T1[B][P];
+  float A[B][P];          // columns, rows in row_at order
+  float V[B][P];          // L^-1 (lower), then columns as A
   float d[B];
   float key[B];
   int drop[B];
   int rank[B];
   unsigned short pairs[(B - 1) * (B / 2)];
-  int flag;
+  float col[2][B], row[2][B];   // of the Cholesky sweep
+  int sweeps;
 };
+
+// C[i][j] = sum over l < n, in order, of X[l][i] Y[l][j], i, j < n, by tiles
+// of R x 4, one thread each (b = 64: 4 x 4, two 16-byte loads for 16 products;
+// b = 32 has too few tiles for that, and takes single rows).
+template <int R, int P, typename F>
+__device__ __forceinline__ void small_product(int n, const float (*X)[P],
+                                              const float (*Y)[P], F put) {
+  const int n4 = (n + 3) / 4, nr = (n + R - 1) / R;
+  for (int e = threadIdx.x; e < nr * n4; e += blockDim.x) {
+    const int i = R * (e / n4), j = 4 * (e % n4);
+    float acc[R][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+#pragma unroll 8
+    for (int l = 0; l < n; ++l) {
+      float x[R], y[4];
+      ld_vec(&X[l][i], x);
+      ld_vec(&Y[l][j], y);
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(x[r], y[c], acc[r][c]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (i + r < n && j + c < n) put(i + r, j + c, acc[r][c]);
+  }
+}
 
 // Launched with 1024 threads, or with 512 (enough for the Jacobi's b / 4
 // warps at b = 64) when there are more blocks than SMs: two such CTAs share
@@ -514,7 +594,7 @@ k_rr_solve(const BlockMeta *__restrict__ meta, SolverState *__restrict__ state,
   const BlockMeta bm = meta[blk];
   const int n = state[blk].bsub;
   const int tid = threadIdx.x;
-  const int lane = tid & 31, wid = tid >> 5, nw = (int)blockDim.x >> 5;
+  const int lane = tid & 31, wid = tid >> 5;
   const int ne = n + (n & 1), np = ne / 2;
   const long long c0 = clock64();
   build_pairs(ne, sm.pairs);
@@ -530,7 +610,7 @@ k_rr_solve(const BlockMeta *__restrict__ meta, SolverState *__restrict__ state,
       h += part[(int64_t)t * 2 * B * B + B * B + i * B + j];
     }
     sm.S[i][j] = s;
-    sm.H[i][j] = h;
+    sm.H[j][i] = h;             // transposed
   }
   __syncthreads();
   // 2. unit diagonal
@@ -548,73 +628,109 @@ k_rr_solve(const BlockMeta *__restrict__ meta, SolverState *__restrict__ state,
   __syncthreads();
   // 3. Cholesky S_n = L L^T, right-looking: for each column j, the pivot
   // S[j][j] already holds S_jj - sum_{l<j} L_jl^2 (subtracted one l at a
-  // time, in order), the column below it is scaled, then every thread
-  // updates its entries of the trailing triangle, S[i][l] -= L_ij L_lj.
-  // This is the same sequence of fused multiply-adds per entry as a
-  // left-looking loop over l, but with O(1) work per thread per column.
+  // time, in order) and the trailing triangle gets S[i][l] -= L_ij L_lj.
   // Weak pivots are dropped: the column is treated as zero below its unit
   // diagonal, so it also changes nothing in the trailing update.
   // 4. L^-1 in the same sweep: Li starts as I; at step j row j is divided by
   // L_jj (it has received all its updates) and then the rows below get
   // Li[i][c] -= L_ij Li[j][c] for c <= j. Per entry these are the fused
   // multiply-adds of forward substitution in the same order (l ascending,
-  // then the division), so the result is bitwise the same, but every step
-  // is parallel over the entries instead of one dependent chain per column.
-  for (int j = 0; j < n; ++j) {
-    const float piv = sm.S[j][j];
-    const bool drop = !(piv > kPivotDrop);
-    const float ljj = drop ? 1.f : __fsqrt_rn(piv);
-    const float inv = __frcp_rn(ljj);
-    for (int i = j + 1 + tid; i < n; i += blockDim.x)
-      sm.S[i][j] = drop ? 0.f : sm.S[i][j] * inv;
-    for (int c = tid; c <= j; c += blockDim.x) sm.Li[j][c] = sm.Li[j][c] / ljj;
-    if (tid == 0) {
-      sm.drop[j] = drop;
-      sm.key[j] = ljj;          // L's diagonal; S[j][j] stays readable
+  // then the division), so every step is parallel over the entries.
+  // Eight warps keep the rows of S and Li in registers (warp w the rows w,
+  // w + 8, ..., lane l the columns l, l + 32); a step's column j of S and row j
+  // of Li go round in shared memory, in one of two buffers, so a step has one
+  // barrier. Every warp takes the root, scales the column and divides the row
+  // for itself; the entries above S's diagonal and the finished rows are
+  // updated too, but never read. A step takes 385 cycles at b = 32 (1,100 with
+  // 32 warps on shared rows, two barriers and a division per entry) and 750 at
+  // b = 64; sixteen warps: 480 and 720, and 1,130 instead of 1,010 with two
+  // CTAs on an SM.
+  constexpr int kCholWarps = 8;
+  constexpr int NC = (B + 31) / 32, NR = (B + kCholWarps - 1) / kCholWarps;
+  if (wid < kCholWarps) {
+    float sr[NR][NC], lr[NR][NC];
+#pragma unroll
+    for (int k = 0; k < NR; ++k)
+#pragma unroll
+      for (int h = 0; h < NC; ++h) {
+        const int i = wid + kCholWarps * k, l = lane + 32 * h;
+        sr[k][h] = i < n && l < n ? sm.S[i][l] : 0.f;
+        lr[k][h] = i == l ? 1.f : 0.f;
+      }
+    for (int i = tid; i < B; i += 32 * kCholWarps) {
+      sm.col[0][i] = i < n ? sm.S[i][0] : 0.f;
+      sm.row[0][i] = i == 0 ? 1.f : 0.f;
     }
-    __syncthreads();
-    // trailing triangle j < l <= i < n: a warp per row, lanes over l
-    for (int i = j + 1 + wid; i < n; i += nw) {
-      const float sij = sm.S[i][j];
-      for (int l = j + 1 + lane; l <= i; l += 32)
-        sm.S[i][l] = fmaf(-sij, sm.S[l][j], sm.S[i][l]);
-      // the row of L^-1, columns 0 .. j
-      for (int c = lane; c <= j; c += 32)
-        sm.Li[i][c] = fmaf(-sij, sm.Li[j][c], sm.Li[i][c]);
+    bar_sync(1, 32 * kCholWarps);
+    for (int j = 0; j < n; ++j) {
+      const int buf = j & 1;
+      const float piv = sm.col[buf][j];
+      float lj[NC], row[NC];               // L_lj and L^-1_jc, l, c by lane
+#pragma unroll
+      for (int h = 0; h < NC; ++h) {
+        lj[h] = sm.col[buf][(lane + 32 * h) % B];
+        row[h] = sm.row[buf][(lane + 32 * h) % B];
+      }
+      const bool drop = !(piv > kPivotDrop);
+      const float ljj = drop ? 1.f : __fsqrt_rn(piv);
+      const float inv = __frcp_rn(ljj);
+#pragma unroll
+      for (int h = 0; h < NC; ++h) {
+        const int l = lane + 32 * h;
+        lj[h] = l > j && !drop ? lj[h] * inv : 0.f;
+        row[h] = l <= j ? quotient(row[h], ljj, inv) : 0.f;
+        if (wid == 0 && l <= j) sm.V[j][l] = row[h];
+      }
+      if (tid == 0) sm.drop[j] = drop;
+      const int nx = j + 1;                // publish column and row nx
+#pragma unroll
+      for (int k = 0; k < NR; ++k) {
+        const int i = wid + kCholWarps * k;
+        // L_ij, 0 for the rows that are done
+        const float sij = __shfl_sync(
+            0xffffffffu, kCholWarps * k < 32 ? lj[0] : lj[NC - 1], i & 31);
+#pragma unroll
+        for (int h = 0; h < NC; ++h) {
+          sr[k][h] = fmaf(-sij, lj[h], sr[k][h]);
+          lr[k][h] = fmaf(-sij, row[h], lr[k][h]);
+        }
+        if (i < B && lane == (nx & 31))
+          sm.col[buf ^ 1][i] = nx < 32 ? sr[k][0] : sr[k][NC - 1];
+        if (i == nx) {
+#pragma unroll
+          for (int h = 0; h < NC; ++h)
+            if (lane + 32 * h < B) sm.row[buf ^ 1][lane + 32 * h] = lr[k][h];
+        }
+      }
+      bar_sync(1, 32 * kCholWarps);
     }
-    __syncthreads();
   }
+  __syncthreads();
   // 5. T1 = D^-1 L^-T, dropped basis columns are zero
   for (int e = tid; e < n * n; e += blockDim.x) {
     const int i = e / n, j = e % n;
     float v = 0.f;
-    if (!sm.drop[j] && sm.d[i] > 0.f) v = sm.Li[j][i] / sm.d[i];
+    if (i <= j && !sm.drop[j] && sm.d[i] > 0.f) v = sm.V[j][i] / sm.d[i];
     sm.T1[i][j] = v;
   }
   __syncthreads();
-  // 6. H' = T1^T H T1 (Li reused as scratch for H T1); A holds H' by
-  // columns (A[j][i] = H'_ij, symmetrised), V = I
-  for (int e = tid; e < n * n; e += blockDim.x) {
-    const int i = e / n, j = e % n;
-    float acc = 0.f;
-    for (int l = 0; l < n; ++l) acc = fmaf(sm.H[i][l], sm.T1[l][j], acc);
-    sm.Li[i][j] = acc;
-  }
+  // 6. H' = T1^T H T1 (Li reused for H T1, S for H'); A holds H' by columns
+  // (A[j] = column j, symmetrised), V = I
+  constexpr int R = B >= 64 ? 4 : 1;
+  small_product<R>(n, sm.H, sm.T1,
+                   [&](int i, int j, float v) { sm.Li[i][j] = v; });
   __syncthreads();
-  for (int e = tid; e < n * n; e += blockDim.x) {
-    const int i = e / n, j = e % n;
-    float acc = 0.f;
-    for (int l = 0; l < n; ++l) acc = fmaf(sm.T1[l][i], sm.Li[l][j], acc);
-    sm.V[i][j] = acc;
-  }
-  __syncthreads();
-  for (int e = tid; e < n * n; e += blockDim.x) {
-    const int i = e / n, j = e % n;
-    sm.A[j][i] = 0.5f * (sm.V[i][j] + sm.V[j][i]);
-  }
-  __syncthreads();
+  small_product<R>(n, sm.T1, sm.Li,
+                   [&](int i, int j, float v) { sm.S[i][j] = v; });
+  // H is free: T1^T for the last product
   for (int e = tid; e < n * n; e += blockDim.x)
-    sm.V[e / n][e % n] = (e / n == e % n) ? 1.f : 0.f;
+    sm.H[e % n][e / n] = sm.T1[e / n][e % n];
+  __syncthreads();
+  for (int e = tid; e < n * B; e += blockDim.x) {
+    const int j = e / B, i = e % B;
+    sm.A[j][row_at<B>(i)] = i < n ? 0.5f * (sm.S[i][j] + sm.S[j][i]) : 0.f;
+    sm.V[j][row_at<B>(i)] = i == j ? 1.f : 0.f;
+  }
   __syncthreads();
   // 7. eigen-decomposition of H' (V by columns: V[j] is eigenvector j)
   const long long c1 = clock64();
@@ -627,13 +743,22 @@ k_rr_solve(const BlockMeta *__restrict__ meta, SolverState *__restrict__ state,
   // test.
   const float tol =
       (state[blk].iters == 0 && n < bm.s) ? kJacobiTolFirst : kJacobiTol;
-  const int sweeps = onesided_jacobi<B>(sm.A, sm.V, n, max_sweeps, sm.pairs,
-                                        &sm.flag, tol);
+  if (wid < (np + 1) / 2) {
+    const int sw =
+        onesided_jacobi<B>(sm.A, sm.V, n, max_sweeps, sm.pairs, tol);
+    if (tid == 0) sm.sweeps = sw;
+  }
+  __syncthreads();
+  const int sweeps = sm.sweeps;
   const long long c2 = clock64();
   // 8. eigenvalues = column norms; descending order, dropped directions last
   for (int j = tid; j < n; j += blockDim.x) {
     float nn = 0.f;
-    for (int r = 0; r < n; ++r) nn = fmaf(sm.A[j][r], sm.A[j][r], nn);
+#pragma unroll 8
+    for (int r = 0; r < n; ++r) {
+      const float v = sm.A[j][row_at<B>(r)];
+      nn = fmaf(v, v, nn);
+    }
     sm.d[j] = sqrtf(nn);                  // d is free after step 5
     sm.key[j] = sm.drop[j] ? -INFINITY : sm.d[j];
   }
@@ -648,17 +773,19 @@ k_rr_solve(const BlockMeta *__restrict__ meta, SolverState *__restrict__ state,
     sm.rank[i] = r;
   }
   __syncthreads();
-  float *Tb = Tout + (int64_t)blk * B * B;
-  for (int e = tid; e < B * B; e += blockDim.x) {
-    const int i = e / B, j = e % B;
-    if (i < n && j < n) {
-      float acc = 0.f;
-      for (int l = 0; l < n; ++l) acc = fmaf(sm.T1[i][l], sm.V[j][l], acc);
-      Tb[i * B + sm.rank[j]] = acc;
-    } else {
-      Tb[i * B + j] = 0.f;
-    }
+  // V^T (rows l, columns by rank) for T = T1 V; zeros past n
+  for (int e = tid; e < n * n; e += blockDim.x) {
+    const int j = e / n, l = e % n;
+    sm.Li[l][sm.rank[j]] = sm.V[j][row_at<B>(l)];
   }
+  float *Tb = Tout + (int64_t)blk * B * B;
+  for (int e = tid; n < B && e < B * B; e += blockDim.x) {
+    const int i = e / B, j = e % B;
+    if (i >= n || j >= n) Tb[e] = 0.f;
+  }
+  __syncthreads();
+  small_product<R>(n, sm.H, sm.Li,
+                   [&](int i, int j, float v) { Tb[i * B + j] = v; });
   for (int i = tid; i < B; i += blockDim.x) {
     if (i < n) theta[(int64_t)blk * B + sm.rank[i]] = sm.drop[i] ? 0.f : sm.d[i];
     else theta[(int64_t)blk * B + i] = 0.f;
@@ -815,7 +942,7 @@ k_check(const BlockMeta *__restrict__ meta, SolverState *__restrict__ state,
         const double *__restrict__ RP, const float *__restrict__ theta,
         float *__restrict__ Finv, int max_iters, int max_degree, float tol,
         int32_t *running) {
-  __shared__ double r2[B], x2[B];
+  __shared__ double r2[B], x2[B], part[256], rel[B];
   __shared__ int s_done;
   const int blk = blockIdx.x;
   pdl_wait();
@@ -825,27 +952,61 @@ k_check(const BlockMeta *__restrict__ meta, SolverState *__restrict__ state,
   const BlockMeta bm = meta[blk];
   const int n = st.bsub, s = bm.s, keff = bm.keff;
   const float *th = theta + (int64_t)blk * B;
-  if (threadIdx.x < B) {
-    double a = 0.0, b = 0.0;
-#pragma unroll 8
-    for (int t = 0; t < bm.nt; ++t) {
-      const double *rp = RP + (int64_t)(bm.t0 + t) * 2 * B;
-      a += rp[threadIdx.x];
-      b += rp[B + threadIdx.x];
+  // The tiles' sums, in float64 (2 B of them): each by 256 / (2 B) threads,
+  // which take every G-th tile, then the threads' sums in order. A float64
+  // operation takes a warp 63 cycles here whether or not it depends on the
+  // last, and a square root or a division about twenty of them, so they are
+  // spread over the threads: with one thread per column, and thread 0 taking
+  // the square roots of the wanted pairs' quotients one after another, the
+  // kernel took 16 us at b = 32, k = 10 and 49 us at b = 64, k = 40 (now 11 and 20 us, most
+  // of it waiting for the kernel before it).
+  {
+    constexpr int G = 256 / (2 * B);
+    const int col = (int)threadIdx.x % (2 * B), g = (int)threadIdx.x / (2 * B);
+    double a = 0.0;
+#pragma unroll 4
+    for (int t = g; t < bm.nt; t += G)
+      a += RP[(int64_t)(bm.t0 + t) * 2 * B + col];
+    part[threadIdx.x] = a;
+    __syncthreads();
+    if (threadIdx.x < 2 * B) {
+#pragma unroll
+      for (int h = 1; h < G; ++h) a += part[threadIdx.x + 2 * B * h];
+      (threadIdx.x < B ? r2 : x2)[col % B] = a;
     }
-    r2[threadIdx.x] = a;
-    x2[threadIdx.x] = b;
+    __syncthreads();
+    // |G x_j - theta_j x_j| / |x_j| of the wanted pairs
+    if (threadIdx.x < B) {
+      const int j = threadIdx.x;
+      rel[j] = j < keff && j < n
+                   ? (x2[j] > 0.0 ? sqrt(r2[j] / x2[j]) : sqrt(r2[j]))
+                   : 0.0;
+    }
   }
   __syncthreads();
+  // their largest, compared as integers (they are not negative; a NaN counts
+  // as 0, as fmax would have it)
+  double worst = 0.0;
+  if (threadIdx.x < 32) {
+    constexpr long long kInf = 0x7ff0000000000000ll;
+    long long w = 0;
+    for (int j = threadIdx.x; j < B; j += 32) {
+      const long long v = __double_as_longlong(rel[j]);
+      if (v <= kInf && v > w) w = v;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long v = __shfl_xor_sync(0xffffffffu, w, o);
+      w = v > w ? v : w;
+    }
+    worst = __longlong_as_double(w);
+  }
   if (threadIdx.x == 0) {
     // The convergence test, in float64: |G x_j - theta_j x_j| / |x_j| <=
     // tol theta_1 for the wanted pairs. For orthonormal Ritz vectors it
     // also bounds the off-diagonal entries |x_i^T G x_j| = |x_i^T r_j| of
     // the Rayleigh quotient matrix by the same amount.
     const float t1 = th[0];
-    double worst = 0.0;
-    for (int j = 0; j < keff && j < n; ++j)
-      worst = fmax(worst, x2[j] > 0.0 ? sqrt(r2[j] / x2[j]) : sqrt(r2[j]));
     const unsigned long long wanted =
         keff >= 64 ? ~0ull : ((1ull << keff) - 1ull);
     st.iters += 1;
