@@ -90,7 +90,8 @@ typedef struct {
     int32_t gram_path;    /* BSVD_FP32 only (the others always use their
                              tensor-core Gram). 0: tensor cores when exact,
                              else FP32 SIMT; 1: FP32 SIMT always; 2: tensor
-                             cores or BSVD_EINVAL from bsvd_factor */
+                             cores, or BSVD_EINVAL from bsvd_factor unless
+                             every offset is whole */
     double tol;           /* residual |G v - theta v| <= tol * theta_1;
                              <= 0: default, 1e-5 for BSVD_FP32, 1e-4 for
                              BSVD_TF32 and 5e-4 for BSVD_BF16 (their Gram
@@ -231,9 +232,9 @@ bsvd_status bsvd_partition_quantile(bsvd_ctx *ctx, int64_t m, int64_t n,
  * its top eigenpairs by Chebyshev-filtered subspace iteration with
  * Rayleigh-Ritz steps solved by Jacobi. Factors stay on the device.
  * With BSVD_FP32 the Gram runs on the tensor cores, exactly, when every
- * rating minus its block's rounded mean is a small integer (integer rating
- * scales), else on the FP32 SIMT pipes; gram_path in the config can force
- * either. BSVD_TF32 and BSVD_BF16 run a single reduced-precision product
+ * rating minus its block's rounded mean is a small multiple of one half (whole
+ * and half-star rating scales), else on the FP32 SIMT pipes; gram_path in the
+ * config can force either (2 takes whole offsets only). BSVD_TF32 and BSVD_BF16 run a single reduced-precision product
  * on the tensor cores.
  * k >= 0; k = 0 keeps no factor (predictions are then the block means).
  * The limit is k <= 56.

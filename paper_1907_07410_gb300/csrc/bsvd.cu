@@ -94,11 +94,11 @@ struct bsvd_ctx {
       d_maxabs, d_mu, d_W, d_err;
   // bf16 [Y; M] planes, per-block shift and delta, TMA maps (tensor Gram)
   bool tc_planes = false, tc_exact = false;
-  // the float32 arena W is written unless the BF16 form's tensor-core
-  // projection reads the bf16 copy instead
+  // the float32 arena W is written unless the tensor-core projection reads
+  // the BF16 form's copy, or rebuilds the cells from the exact Gram's planes
   bool w32 = true;
   int32_t gram_used = 0;    // 1: FP32 SIMT, 2: exact tensor, 3: tf32, 4: bf16
-  DevBuf d_VX, d_shift, d_delta, d_maps, d_flag;
+  DevBuf d_VX, d_shift, d_delta, d_maps;
   DevBuf d_wmaps;           // TMA maps over the float32 blocks (tf32 Gram)
 
   // factor
@@ -240,11 +240,16 @@ cudaError_t device_view(bsvd_ctx *c, const void *ptr, size_t bytes,
   return e;
 }
 
-bsvd_status read_errors(bsvd_ctx *c, const char *what) {
-  int32_t h = 0;
-  CK(cudaMemcpyAsync(&h, c->d_err.p, sizeof h, cudaMemcpyDeviceToHost, c->st),
-     what);
+// The error word, as a status; the word beside it (what the planes' scatter
+// found) to *flag when asked.
+bsvd_status read_errors(bsvd_ctx *c, const char *what,
+                        int32_t *flag = nullptr) {
+  int32_t both[2] = {0, 0};
+  CK(cudaMemcpyAsync(both, c->d_err.p, sizeof(int32_t) * (flag ? 2 : 1),
+                     cudaMemcpyDeviceToHost, c->st), what);
   CK(cudaStreamSynchronize(c->st), what);
+  const int32_t h = both[0];
+  if (flag) *flag = both[1];
   if (h) {
     std::string msg = std::string(what) + ":";
     if (h & kErrIndex) msg += " id out of range or off the block diagonal;";
@@ -534,8 +539,9 @@ bsvd_status bsvd_create(const bsvd_config *cfg, bsvd_ctx **out) {
   if (cudaGetDevice(&c->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount,
                              c->device) != cudaSuccess ||
-      c->d_err.ensure(sizeof(int32_t)) != cudaSuccess ||
-      cudaMemsetAsync(c->d_err.p, 0, sizeof(int32_t), c->st) != cudaSuccess ||
+      c->d_err.ensure(2 * sizeof(int32_t)) != cudaSuccess ||
+      cudaMemsetAsync(c->d_err.p, 0, 2 * sizeof(int32_t), c->st) !=
+          cudaSuccess ||
       cudaStreamSynchronize(c->st) != cudaSuccess) {
     cudaGetLastError();
     delete c;
@@ -562,7 +568,7 @@ void bsvd_destroy(bsvd_ctx *c) {
                     &c->d_FL, &c->d_sigma, &c->d_running, &c->d_gtiles,
                     &c->d_rowtiles, &c->d_ltiles, &c->s_a, &c->s_b, &c->s_c,
                     &c->s_out, &c->d_partials, &c->d_rmse, &c->d_VX,
-                    &c->d_shift, &c->d_delta, &c->d_maps, &c->d_flag,
+                    &c->d_shift, &c->d_delta, &c->d_maps,
                     &c->d_wmaps, &c->d_ptiles, &c->d_gmaps, &c->d_xmaps, &c->d_XB, &c->d_ZB,
                     &c->d_pjtiles, &c->d_pwmaps, &c->d_state0,
                     &c->d_sgd_key[0], &c->d_sgd_key[1], &c->d_sgd_src[0],
@@ -682,9 +688,10 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
   CK(c->d_sums.ensure(sizeof(long long) * nb), "partition");
   CK(c->d_maxabs.ensure(sizeof(unsigned int)), "partition");
   CK(c->d_mu.ensure(sizeof(float) * nb), "partition");
-  c->w32 = !(c->cfg.precision == BSVD_BF16 && c->cfg.panel_path == 0);
-  if (c->w32)
-    CK(c->d_W.ensure(sizeof(float) * std::max<int64_t>(off, 1)), "partition");
+  c->tc_planes = c->cfg.gram_path != 1 && c->cfg.precision == BSVD_FP32;
+  // with planes, W is written only after they turn out not to do
+  c->w32 = c->cfg.panel_path == 1 ||
+           (c->cfg.precision != BSVD_BF16 && !c->tc_planes);
   CK(cudaMemcpyAsync(c->d_rb.p, c->rb.data(), sizeof(int64_t) * (p + 1),
                      cudaMemcpyHostToDevice, c->st), "partition");
   CK(cudaMemcpyAsync(c->d_cb.p, c->cb.data(), sizeof(int64_t) * (q + 1),
@@ -695,7 +702,7 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
   // permutations: copied into context memory, then checked on the device
   c->has_rperm = row_perm != nullptr;
   c->has_cperm = col_perm != nullptr;
-  CK(cudaMemsetAsync(c->d_err.p, 0, sizeof(int32_t), c->st), "partition");
+  CK(cudaMemsetAsync(c->d_err.p, 0, 2 * sizeof(int32_t), c->st), "partition");
   if (row_perm) {
     CK(c->d_rperm.ensure(sizeof(int32_t) * m), "partition");
     CK(c->d_seen.ensure(sizeof(int32_t) * std::max(m, n)), "partition");
@@ -730,10 +737,18 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
      "partition");
   CK(cudaMemsetAsync(c->d_maxabs.p, 0, sizeof(unsigned int), c->st),
      "partition");
-  if (c->w32)
+  const GridDesc g = c->grid();
+  auto write_w = [&]() -> bsvd_status {
+    CK(c->d_W.ensure(sizeof(float) * std::max<int64_t>(off, 1)), "partition");
     CK(cudaMemsetAsync(c->d_W.p, 0, sizeof(float) * std::max<int64_t>(off, 1),
                        c->st), "partition");
-  const GridDesc g = c->grid();
+    CK(launch_scatter(g, c->d_meta.as<BlockMeta>(), nnz, (const int32_t *)du,
+                      (const int32_t *)di, (const float *)dx,
+                      c->d_mu.as<float>(), c->d_W.as<float>(), c->st),
+       "partition: scatter");
+    c->launches += nnz > 0;
+    return BSVD_OK;
+  };
   std::fill(c->phase_ms, c->phase_ms + 8, 0.0);
   mark(c, 0);
   CK(launch_count(g, nnz, (const int32_t *)du, (const int32_t *)di,
@@ -744,51 +759,57 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
                   c->d_sums.as<long long>(), c->d_maxabs.as<unsigned int>(),
                   c->d_mu.as<float>(), c->d_err.as<int32_t>(), c->st),
      "partition: means");
-  __nv_bfloat16 *wh = nullptr;
+  c->launches += nnz > 0 ? 2 : 1;
+  if (c->w32) {
+    const bsvd_status ws = write_w();
+    if (ws != BSVD_OK) return ws;
+  }
   if (c->cfg.precision == BSVD_BF16) {
     CK(c->d_VX.ensure(2 * std::max<int64_t>(vxoff, 1)), "partition");
     CK(cudaMemsetAsync(c->d_VX.p, 0, 2 * std::max<int64_t>(vxoff, 1), c->st),
        "partition");
-    wh = c->d_VX.as<__nv_bfloat16>();
+    CK(launch_scatter_bf16(g, c->d_meta.as<BlockMeta>(), nnz,
+                           (const int32_t *)du, (const int32_t *)di,
+                           (const float *)dx, c->d_mu.as<float>(),
+                           c->d_VX.as<__nv_bfloat16>(), c->st),
+       "partition: scatter");
+    c->launches += nnz > 0;
   }
-  CK(launch_scatter(g, c->d_meta.as<BlockMeta>(), nnz, (const int32_t *)du,
-                    (const int32_t *)di, (const float *)dx,
-                    c->d_mu.as<float>(), c->w32 ? c->d_W.as<float>() : nullptr,
-                    wh, c->st),
-     "partition: scatter");
-  c->launches += nnz > 0 ? 3 : 1;
   // bf16 planes for the exact tensor-core Gram
-  c->tc_planes = c->cfg.gram_path != 1 && c->cfg.precision == BSVD_FP32;
   c->tc_exact = false;
   if (c->tc_planes) {
     CK(c->d_VX.ensure(2 * std::max<int64_t>(vxoff, 1)), "partition");
     CK(c->d_shift.ensure(sizeof(float) * nb), "partition");
     CK(c->d_delta.ensure(sizeof(float) * nb), "partition");
-    CK(c->d_flag.ensure(sizeof(int32_t)), "partition");
     CK(cudaMemsetAsync(c->d_VX.p, 0, 2 * std::max<int64_t>(vxoff, 1), c->st),
        "partition");
-    CK(cudaMemsetAsync(c->d_flag.p, 0, sizeof(int32_t), c->st), "partition");
     CK(launch_plane_shift(nb, c->d_counts.as<unsigned long long>(),
                           c->d_sums.as<long long>(), c->d_shift.as<float>(),
                           c->d_delta.as<float>(), c->st), "partition: shift");
     CK(launch_scatter_planes(g, c->d_meta.as<BlockMeta>(), nnz,
                              (const int32_t *)du, (const int32_t *)di,
                              (const float *)dx, c->d_shift.as<float>(),
-                             c->d_VX.as<__nv_bfloat16>(), c->d_flag.as<int32_t>(),
+                             c->d_VX.as<__nv_bfloat16>(), c->d_err.as<int32_t>() + 1,
                              c->st), "partition: planes");
     c->launches += nnz > 0 ? 2 : 1;
   }
   mark(c, 1);
-  bsvd_status s = read_errors(c, "partition");
+  int32_t flag = 0;
+  bsvd_status s = read_errors(c, "partition", &flag);
   if (s != BSVD_OK) return s;
-  take(c, 0, 0, 1);
   if (c->tc_planes) {
-    int32_t flag = 0;
-    CK(cudaMemcpyAsync(&flag, c->d_flag.p, sizeof flag, cudaMemcpyDeviceToHost,
-                       c->st), "partition");
-    CK(cudaStreamSynchronize(c->st), "partition");
-    c->tc_exact = (flag & kErrNotExact) == 0;
+    // gram_path 2 takes whole ratings only; by default halves are exact too
+    c->tc_exact = (flag & kErrNotExact) == 0 ||
+                  (c->cfg.gram_path == 0 && (flag & kErrNotHalf) == 0);
+    if (!c->w32 && (!c->tc_exact || (flag & kErrNotRebuilt) != 0)) {
+      c->w32 = true;
+      s = write_w();
+      if (s != BSVD_OK) return s;
+      mark(c, 1);
+      CK(cudaStreamSynchronize(c->st), "partition");
+    }
   }
+  take(c, 0, 0, 1);
   if ((c->tc_planes && c->tc_exact) || c->cfg.precision == BSVD_BF16) {
     const int64_t plane_rows = c->cfg.precision == BSVD_BF16 ? 1 : 2;
     {
@@ -1186,7 +1207,7 @@ static bsvd_status factor_impl(bsvd_ctx *c, int32_t k, const int32_t *ks) {
       sig.insert(sig.end(), b, b + n);
     };
     put(c->meta.data(), sizeof(BlockMeta) * nb);
-    const int64_t head[4] = {B, kp, panel_tc ? 1 : 0, nb};
+    const int64_t head[5] = {B, kp, panel_tc ? 1 : 0, nb, c->w32 ? 1 : 0};
     put(head, sizeof head);
     const void *ptrs[] = {c->d_G.p, c->d_W.p, c->d_XB.p, c->d_ZB.p,
                           c->d_gtiles.p, c->d_rowtiles.p, c->d_ltiles.p,
@@ -1286,19 +1307,25 @@ static bsvd_status factor_impl(bsvd_ctx *c, int32_t k, const int32_t *ks) {
                        sizeof(CUtensorMap) * 2 * nb, cudaMemcpyHostToDevice,
                        c->st), "factor");
     // the tensor-core projection F_L = W^T F_s: one TMA map per block over
-    // W (s_pad rows x L_pad columns, float32, boxes of 32 rows x 128
-    // columns, plain layout) and 128-column tiles
+    // W (s_pad rows x L_pad columns, float32), or without W over its planes
+    // (2 s128 rows, bf16): boxes of 32 rows x 128 columns, plain layout
     c->h_pwmaps.assign(nb, CUtensorMap());
     std::memset(c->h_pwmaps.data(), 0, sizeof(CUtensorMap) * nb);
     for (int32_t b = 0; b < nb && !proj16; ++b) {
       const BlockMeta &bm = c->meta[b];
       if (bm.s == 0 || bm.L == 0 || !bm.owned) continue;
-      cuuint64_t dims[2] = {(cuuint64_t)bm.L_pad, (cuuint64_t)bm.s_pad};
-      cuuint64_t strides[1] = {(cuuint64_t)bm.L_pad * 4};
+      const int esize = c->w32 ? 4 : 2;
+      cuuint64_t dims[2] = {(cuuint64_t)bm.L_pad,
+                            (cuuint64_t)(c->w32 ? bm.s_pad : 2 * bm.s128)};
+      cuuint64_t strides[1] = {(cuuint64_t)bm.L_pad * esize};
       cuuint32_t box[2] = {128, 32};
       cuuint32_t es[2] = {1, 1};
-      CUresult r = enc(&c->h_pwmaps[b], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                       c->d_W.as<float>() + bm.w_off, dims, strides, box, es,
+      void *base = c->w32 ? (void *)(c->d_W.as<float>() + bm.w_off)
+                          : (void *)(c->d_VX.as<__nv_bfloat16>() + bm.vx_off);
+      CUresult r = enc(&c->h_pwmaps[b],
+                       c->w32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                              : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                       base, dims, strides, box, es,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                        CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -1516,7 +1543,8 @@ static bsvd_status factor_impl(bsvd_ctx *c, int32_t k, const int32_t *ks) {
         if ((r = launch_project_tc(B, e.meta, c->d_pjtiles.as<int2>(),
                                    c->n_pjtiles, c->d_pwmaps.as<CUtensorMap>(),
                                    c->d_xmaps.as<CUtensorMap>(),
-                                   c->d_FL.as<float>(), kp,
+                                   c->w32 ? nullptr : c->d_shift.as<float>(),
+                                   c->d_mu.as<float>(), c->d_FL.as<float>(), kp,
                                    c->d_err.as<int32_t>(), c->st)) !=
             cudaSuccess)
           return r;
@@ -1558,7 +1586,8 @@ static bsvd_status factor_impl(bsvd_ctx *c, int32_t k, const int32_t *ks) {
                             c->d_theta.p, c->d_Fs.p, c->d_FL.p, c->d_sigma.p,
                             c->d_running.p, c->d_err.p, c->d_maps.p,
                             c->d_delta.p, c->d_wmaps.p, c->d_pctl.p,
-                            c->d_ptime.p, c->d_loopctl.p, c->d_finv.p};
+                            c->d_ptime.p, c->d_loopctl.p, c->d_finv.p,
+                            c->d_shift.p, c->d_mu.p};
       const unsigned char *pb = reinterpret_cast<const unsigned char *>(bufs);
       key.insert(key.end(), pb, pb + sizeof bufs);
       c->gkey_now.swap(key);
@@ -1850,6 +1879,28 @@ bsvd_status bsvd_get_block(bsvd_ctx *c, int32_t b, int32_t *mb, int32_t *nb,
     CK(cudaMemcpyAsync(W.data(), c->d_W.as<float>() + bm.w_off,
                        sizeof(float) * W.size(), cudaMemcpyDeviceToHost, c->st),
        "get_block");
+  } else if (dense && c->tc_planes) {
+    // the exact Gram's planes: the cells as the projection rebuilds them
+    const size_t n = (size_t)bm.s_pad * bm.L_pad;
+    std::vector<__nv_bfloat16> Mh(n);
+    float shift = 0.f, mean = 0.f;
+    Wh.resize(n);
+    W.resize(n);
+    const __nv_bfloat16 *vx = c->d_VX.as<__nv_bfloat16>() + bm.vx_off;
+    CK(cudaMemcpyAsync(Wh.data(), vx, sizeof(__nv_bfloat16) * n,
+                       cudaMemcpyDeviceToHost, c->st), "get_block");
+    CK(cudaMemcpyAsync(Mh.data(), vx + (size_t)bm.s128 * bm.L_pad,
+                       sizeof(__nv_bfloat16) * n, cudaMemcpyDeviceToHost,
+                       c->st), "get_block");
+    CK(cudaMemcpyAsync(&shift, c->d_shift.as<float>() + b, sizeof shift,
+                       cudaMemcpyDeviceToHost, c->st), "get_block");
+    CK(cudaMemcpyAsync(&mean, c->d_mu.as<float>() + b, sizeof mean,
+                       cudaMemcpyDeviceToHost, c->st), "get_block");
+    CK(cudaStreamSynchronize(c->st), "get_block");
+    for (size_t j = 0; j < n; ++j) {
+      const volatile float x = __bfloat162float(Wh[j]) + shift;
+      W[j] = __bfloat162float(Mh[j]) != 0.f ? x - mean : 0.f;
+    }
   } else if (dense) {
     // the BF16 form keeps only the bf16 copy of its blocks
     Wh.resize((size_t)bm.s_pad * bm.L_pad);

@@ -152,7 +152,9 @@ enum : int32_t {
   kErrSumRange = 4,     // count * max|x| >= 2^31 in some block
   kErrBadPerm = 8,      // a permutation entry out of range or repeated
   kErrTimeout = 16,     // a bounded device-side wait gave up
-  kErrNotExact = 32     // a rating is not an exact small integer offset
+  kErrNotExact = 32,    // a rating is not an exact small integer offset
+  kErrNotHalf = 64,     // nor a small multiple of one half
+  kErrNotRebuilt = 128  // a rating is not its offset plus the shift
 };
 
 // Grid description used by every kernel that maps (user, item) to a block.
@@ -208,10 +210,51 @@ __device__ __forceinline__ bool locate(const GridDesc &g, int32_t u,
   return true;
 }
 
-// (r, c) of B -> (a, l) of W: a on the Gram side, l on the reduction side.
-__device__ __forceinline__ void to_w(const BlockMeta &bm, int32_t r,
-                                     int32_t c, int32_t *a, int32_t *l) {
-  if (bm.trans) { *a = c; *l = r; } else { *a = r; *l = c; }
+// A CTA's copy of a grid's bounds, for kernels that look up a block per rating
+// or query: at most kTableBounds bounds a side and kTableBlocks blocks (of
+// which the kernels keep what they need beside it). A larger grid is read in
+// place.
+constexpr int kTableBlocks = 512;
+constexpr int kTableBounds = 512;
+
+struct BoundsTable {
+  int32_t rb[kTableBounds + 1], cb[kTableBounds + 1];
+  // Every thread of the CTA; a barrier has to follow.
+  __device__ __forceinline__ void fill(const GridDesc &g) {
+    for (int j = threadIdx.x; j <= g.p; j += blockDim.x)
+      rb[j] = (int32_t)g.row_bounds[j];
+    for (int j = threadIdx.x; j <= g.q; j += blockDim.x)
+      cb[j] = (int32_t)g.col_bounds[j];
+  }
+};
+inline int32_t grid_blocks(const GridDesc &g) {
+  return g.diag ? g.p : g.p * g.q;
+}
+inline bool fits_table(const GridDesc &g) {
+  return g.p <= kTableBounds && g.q <= kTableBounds &&
+         grid_blocks(g) <= kTableBlocks;
+}
+
+// The block of (u, i) and the positions of u and i (locate, with the bounds
+// from the table); false: an id is out of range or off the block diagonal.
+template <bool TABLE>
+__device__ __forceinline__ bool find_block(const GridDesc &g,
+                                           const BoundsTable &tb, int32_t u,
+                                           int32_t i, int32_t *blk,
+                                           int32_t *ru, int32_t *ci) {
+  if (u < 0 || (int64_t)u >= g.m || i < 0 || (int64_t)i >= g.n) return false;
+  *ru = g.row_perm ? __ldg(g.row_perm + u) : u;
+  *ci = g.col_perm ? __ldg(g.col_perm + i) : i;
+  int32_t bi, bj;
+  if (g.equal_rows) bi = (int32_t)((uint32_t)*ru / (uint32_t)g.br);
+  else if (TABLE) bi = upper_index(tb.rb, g.p, *ru);
+  else bi = upper_index(g.row_bounds, g.p, (int64_t)*ru);
+  if (g.equal_cols) bj = (int32_t)((uint32_t)*ci / (uint32_t)g.bc);
+  else if (TABLE) bj = upper_index(tb.cb, g.q, *ci);
+  else bj = upper_index(g.col_bounds, g.q, (int64_t)*ci);
+  if (g.diag && bi != bj) return false;
+  *blk = g.diag ? bi : bi * g.q + bj;
+  return true;
 }
 
 }  // namespace bsvd

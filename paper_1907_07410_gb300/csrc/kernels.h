@@ -20,11 +20,17 @@ cudaError_t launch_means(int32_t nblocks, const unsigned long long *counts,
                          const long long *sums,
                          const unsigned int *maxabs_bits, float *mu,
                          int32_t *err, cudaStream_t st);
-// W (float32 arena) and Wh (bf16 copy) are each written when not null.
+// Centred cells into the zeroed float32 arena, or their bf16 rounding into the
+// zeroed bf16 blocks.
 cudaError_t launch_scatter(const GridDesc &g, const BlockMeta *meta,
                            int64_t nnz, const int32_t *u, const int32_t *i,
                            const float *x, const float *mu, float *W,
-                           __nv_bfloat16 *Wh, cudaStream_t st);
+                           cudaStream_t st);
+cudaError_t launch_scatter_bf16(const GridDesc &g, const BlockMeta *meta,
+                                int64_t nnz, const int32_t *u,
+                                const int32_t *i, const float *x,
+                                const float *mu, __nv_bfloat16 *Wh,
+                                cudaStream_t st);
 
 // ---- activity-quantile cut of one side (kernels_grid.cu) ----------------
 // Keys are padded to quantile_cut_padded(size) entries. counts: size,
@@ -69,9 +75,12 @@ cudaError_t launch_gram_bf16(const BlockMeta *meta, const int4 *tiles,
 cudaError_t launch_plane_shift(int32_t nblocks, const unsigned long long *counts,
                                const long long *sums, float *shift,
                                float *delta, cudaStream_t st);
-// Y = x - shift, M = 1 at every rating, into the zeroed planes; sets
-// kErrNotExact in *flag when some x - shift is not an integer small enough
-// (|y|^2 L_pad < 2^24, |y| <= 256) for the tensor-core Gram to be exact.
+// Y = x - shift, M = 1 at every rating, into the zeroed planes. *flag gets
+// kErrNotExact when some x - shift is not an integer small enough
+// (|y|^2 L_pad < 2^24, |y| <= 256) for the tensor-core Gram to be exact,
+// kErrNotHalf when some is not a multiple of one half small enough
+// (4 |y|^2 L_pad < 2^24, |y| <= 128), kErrNotRebuilt when some rating is not
+// fl32(y + shift).
 cudaError_t launch_scatter_planes(const GridDesc &g, const BlockMeta *meta,
                                   int64_t nnz, const int32_t *u,
                                   const int32_t *i, const float *x,
@@ -130,7 +139,8 @@ cudaError_t launch_gpanel_tc(int32_t bsub, const BlockMeta *meta,
 cudaError_t launch_project_tc(int32_t bsub, const BlockMeta *meta,
                               const int2 *tiles, int32_t ntiles,
                               const CUtensorMap *wmaps,
-                              const CUtensorMap *fmaps, float *FL, int32_t kp,
+                              const CUtensorMap *fmaps, const float *shift,
+                              const float *mu, float *FL, int32_t kp,
                               int32_t *err, cudaStream_t st);
 // B form of F_s (s_pad x kp per block, at fs_off) at 2 x_off of out_bf, in
 // the panel layout with bsub columns (zero past kp); tiles as for the

