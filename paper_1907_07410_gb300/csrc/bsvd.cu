@@ -125,9 +125,10 @@ struct bsvd_ctx {
   // the persistent panel products' tile counter, and the CTAs they launch
   DevBuf d_pctl;
   int32_t nsm = 1;
-  // panel products' device time: [0] summed launch durations (ns), [1] the
-  // running launch's start; the graph loop's step counter
+  // panel products: [0] launches, then (profile = 1) the starts and the ends
+  // of the first nspans of them; the graph loop's step counter
   DevBuf d_ptime, d_loopctl;
+  int32_t nspans = 0;
   // the device-driven form: the captured graph, the layout key it was built
   // for, the key of this and of the previous factorisation, kernel counts
   cudaGraphExec_t gexec = nullptr;
@@ -298,13 +299,15 @@ int32_t subspace_width(int32_t k, int32_t oversample) {
   return 64;
 }
 
-// The panel products' device timer: no time summed yet, no launch running.
+// The panel products' launch count and spans: none yet.
 cudaError_t reset_ptime(bsvd_ctx *c) {
-  cudaError_t e = cudaMemsetAsync(c->d_ptime.p, 0,
-                                  3 * sizeof(unsigned long long), c->st);
+  const size_t w = sizeof(unsigned long long);
+  unsigned long long *p = c->d_ptime.as<unsigned long long>();
+  cudaError_t e = cudaMemsetAsync(p, 0, w, c->st);
+  if (e != cudaSuccess || c->nspans == 0) return e;
+  e = cudaMemsetAsync(p + 1, 0xFF, w * c->nspans, c->st);
   if (e != cudaSuccess) return e;
-  return cudaMemsetAsync(c->d_ptime.as<unsigned long long>() + 1, 0xFF,
-                         sizeof(unsigned long long), c->st);
+  return cudaMemsetAsync(p + 1 + c->nspans, 0, w * c->nspans, c->st);
 }
 
 // Capture one factorisation into c->gexec: pre, then a conditional WHILE
@@ -1178,7 +1181,14 @@ static bsvd_status factor_impl(bsvd_ctx *c, int32_t k, const int32_t *ks) {
   CK(c->d_flip.ensure((size_t)kp * std::max(nb, 1)), "factor");
   CK(c->d_pctl.ensure(2 * sizeof(int32_t)), "factor");
   CK(cudaMemsetAsync(c->d_pctl.p, 0, 2 * sizeof(int32_t), c->st), "factor");
-  CK(c->d_ptime.ensure(3 * sizeof(unsigned long long)), "factor");
+  // every launch of a factorisation (at most 65,536) has a span
+  c->nspans = c->cfg.profile
+                  ? (int32_t)std::min<int64_t>(
+                        ((int64_t)c->cfg.max_iters + 3) *
+                            (c->cfg.cheb_degree + 1) + 2, 65536)
+                  : 0;
+  CK(c->d_ptime.ensure(sizeof(unsigned long long) * (1 + 2 * c->nspans)),
+     "factor");
   CK(c->d_loopctl.ensure(2 * sizeof(int32_t)), "factor");
   const bool tc_maps = panel_tc && !pt.empty();
   if (tc_maps) {
@@ -1413,19 +1423,24 @@ static bsvd_status factor_impl(bsvd_ctx *c, int32_t k, const int32_t *ks) {
     const int2 *rtd = c->d_rowtiles.as<int2>();
     const int nrt = c->n_rowtiles;
     // out = alpha G in + beta in + gamma in2 (see launch_gpanel). The
-    // tensor-core path reads the B form of `in` and writes that of `out`.
+    // tensor-core path reads the B forms of `in` and in2 and writes that of
+    // `out`, except of a plain product's.
     auto panel = [&](int mode, int step, int deg, const float *in,
                      const float *in2, float *out) -> cudaError_t {
       if (panel_tc) {
         const CUtensorMap *xm = c->d_xmaps.as<CUtensorMap>() +
                                 (in == e.X ? 0 : (size_t)nb);
-        float *out_bf = out == e.X ? c->d_XB.as<float>() : c->d_ZB.as<float>();
+        auto bform = [&](const float *p) {
+          return !p ? nullptr
+                    : p == e.X ? c->d_XB.as<float>() : c->d_ZB.as<float>();
+        };
         return launch_gpanel_tc(B, e.meta, e.state, c->d_ptiles.as<int2>(),
                                 c->n_ptiles, c->nsm, c->d_pctl.as<int32_t>(),
-                                c->d_ptime.as<unsigned long long>(),
-                                c->d_gmaps.as<CUtensorMap>(), xm, in, in2, out,
-                                out_bf, mode, step, c->d_err.as<int32_t>(),
-                                c->st);
+                                c->d_ptime.as<unsigned long long>(), c->nspans,
+                                c->d_gmaps.as<CUtensorMap>(), xm, bform(in),
+                                bform(in2), out,
+                                mode == 0 ? nullptr : bform(out), mode, step,
+                                c->d_err.as<int32_t>(), c->st);
       }
       return launch_gpanel(e, rtd, nrt, mode, step, deg, in, in2, out, c->st);
     };
@@ -1682,16 +1697,25 @@ static bsvd_status factor_impl(bsvd_ctx *c, int32_t k, const int32_t *ks) {
     {
       // the panel products' own time (summed over launches on the device),
       // and in graph form the loop's kernel count
-      unsigned long long pt[3] = {0, 0, 0};
+      std::vector<unsigned long long> pt(1 + 2 * (size_t)c->nspans, 0);
       int32_t loops[2] = {0, 0};
-      CK(cudaMemcpyAsync(pt, c->d_ptime.p, sizeof pt, cudaMemcpyDeviceToHost,
-                         c->st), "factor");
+      CK(cudaMemcpyAsync(pt.data(), c->d_ptime.p,
+                         sizeof(unsigned long long) * pt.size(),
+                         cudaMemcpyDeviceToHost, c->st), "factor");
       if (ran_graph)
         CK(cudaMemcpyAsync(loops, c->d_loopctl.p, sizeof loops,
                            cudaMemcpyDeviceToHost, c->st), "factor");
       CK(cudaStreamSynchronize(c->st), "factor");
-      c->phase_ms[5] = (double)pt[0] * 1e-6;
-      c->panel_launches = (int64_t)pt[2];
+      c->panel_launches = (int64_t)pt[0];
+      // each launch's span, first CTA's start to last CTA's end (the two
+      // dies' timers may differ by a little: a negative span of a very short
+      // launch counts as 0)
+      unsigned long long ns = 0;
+      for (int64_t l = 0; l < std::min<int64_t>(pt[0], c->nspans); ++l) {
+        const unsigned long long t0 = pt[1 + l], t1 = pt[1 + c->nspans + l];
+        if (t0 != ~0ull && t1 > t0) ns += t1 - t0;
+      }
+      c->phase_ms[5] = (double)ns * 1e-6;
       // loop steps times their unconditional kernels, plus the filter
       // steps the loop control opened
       if (ran_graph)

@@ -117,19 +117,21 @@ struct EigBuffers {
 // boxes, 128-byte swizzle). The B form of a panel P (s_pad x bsub) sits at
 // 2 x_off: for each 32-row chunk, bsub rows of hi(P) then bsub rows of
 // lo(P), 32 floats each (hi = P rounded to 10 mantissa bits, lo = P - hi).
-// out_bf (optional) receives the B form of `out`.
+// in_bf, in2_bf: the B forms of the inputs (in2_bf for mode 2). out_bf (not
+// for mode 0's result, which nothing multiplies again) receives the B form
+// of the result, out its rows in mode 0 and in a block's last filter step.
 // Persistent: nctas CTAs (one per SM) take the tiles of the running blocks
 // from the counter ctl[0] (ctl: 2 ints, zero before the first launch; the
-// kernel leaves them zero). ptime[0] gains the launch's span in ns (first
-// CTA start to last CTA end), ptime[2] counts launches; ptime[1] must hold
-// ~0 before the first launch (the kernel leaves it so).
+// kernel leaves them zero). ptime[0] counts launches; the start and the end
+// (GPU timer, ns) of the first nspans launches go to ptime[1 + l] and
+// ptime[1 + nspans + l], which must hold ~0 and 0 before.
 cudaError_t launch_gpanel_tc(int32_t bsub, const BlockMeta *meta,
                              SolverState *state, const int2 *tiles,
                              int32_t ntiles, int32_t nctas, int32_t *ctl,
-                             unsigned long long *ptime,
+                             unsigned long long *ptime, int32_t nspans,
                              const CUtensorMap *gmaps,
-                             const CUtensorMap *xmaps, const float *in,
-                             const float *in2, float *out, float *out_bf,
+                             const CUtensorMap *xmaps, const float *in_bf,
+                             const float *in2_bf, float *out, float *out_bf,
                              int mode, int step, int32_t *err,
                              cudaStream_t st);
 // F_L = W^T F_s on the tensor cores (three tf32 passes): tiles are (block,

@@ -159,20 +159,24 @@ __device__ __forceinline__ uint32_t sw128(int r, int c) {
 }
 
 // Sum of the R accumulators' 16 columns at `col`, in a fixed order:
-// (a0 + a1) + (a2 + a3), or a0 + a1.
+// (a0 + a1) + (a2 + a3), or a0 + a1, two loads at a time.
 template <int B>
 __device__ __forceinline__ void acc_sum(uint32_t taddr, uint32_t col,
                                         float (&v)[16]) {
   using L = PanelTc<B>;
   float t[16];
-  tc::tmem_ld16(taddr + col, v);
-  tc::tmem_ld16(taddr + col + 2 * B, t);
+  tc::tmem_ld16_start(taddr + col, v);
+  tc::tmem_ld16_start(taddr + col + 2 * B, t);
+  tc::tmem_wait_ld16(v);
+  tc::tmem_wait_ld16(t);
 #pragma unroll
   for (int j = 0; j < 16; ++j) v[j] += t[j];
   if constexpr (L::R == 4) {
     float u[16];
-    tc::tmem_ld16(taddr + col + 4 * B, u);
-    tc::tmem_ld16(taddr + col + 6 * B, t);
+    tc::tmem_ld16_start(taddr + col + 4 * B, u);
+    tc::tmem_ld16_start(taddr + col + 6 * B, t);
+    tc::tmem_wait_ld16(u);
+    tc::tmem_wait_ld16(t);
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] += u[j] + t[j];
   }
@@ -236,22 +240,39 @@ constexpr size_t panel_ring_smem() {
 
 // Persistent: one CTA per SM. CTA i starts with tile i (if its block is
 // still iterating), then takes tiles from gridDim.x on from a shared
-// counter (ctl[0]; ctl[1] counts finished CTAs, and the last one resets
-// both for the next launch). A claimed tile of an idle block moves the
-// counter past the rest of that block. Warp 0 claims tiles, publishes their
-// indices in a small ring (tq) and loads their G stages; warp kBWarp loads
-// the matching B stages; warps 2 + kPConv .. + 3 run the epilogue. The stage, A-slot and tile counters run on across
-// tiles, so a CTA sets up its barriers and tensor memory once per launch
-// and the loads of the next tile overlap the epilogue of the last. The MMA
-// warp starts a tile only after the epilogue warps have read the previous
-// tile's accumulators (accfree).
+// counter (ctl[0]; ctl[1] counts the CTAs that claim no more, and the last
+// one resets both for the next launch). A claimed tile of an idle block moves
+// the counter past the rest of that block. Warp 0 claims tiles, publishes
+// their indices in a small ring (tq) and loads their G stages; warp kBWarp
+// loads the matching B stages; warps 2 + kPConv .. + 3 run the epilogue. The
+// stage, A-slot and tile counters run on across tiles, so a CTA sets up its
+// barriers and tensor memory once per launch and the loads of the next tile
+// overlap the epilogue of the last. The MMA warp starts a tile only after the
+// epilogue warps have read the previous tile's accumulators (accfree).
+//
+// The launch overlaps the previous kernel's end (pdl_wait), and G does not
+// change in the meantime: the first stages of tile i are loaded before the
+// wait, its first B stages right after it, without looking whether the block
+// still runs. If it does not, kSkip goes through the ring and the roles drain
+// those stages. A product of 16 blocks of about 1,000 rows at b = 32 is some
+// 16 stages of 1,100 cycles in each CTA (load-bound), and took 36,000: the
+// first stage came 4,500 cycles after the wait, behind the look-ups of the
+// tile, the state and the metadata; the epilogue took 12,000, reading strided
+// rows of in and in2 where it used them and writing rows nobody reads; and
+// each CTA ended on the round trips of two counters (2,300). Now: 14.2 us a
+// product, from 18.1 (b = 64, 16 blocks of 1,500 rows: 29.7 from 35.3; b = 64,
+// 256 blocks: 713 from 752; b = 16, 4 blocks: 7.8 from 11.3).
+
+constexpr int kSkip = -2;
+
 template <int B>
 __global__ void __launch_bounds__(kPThreads, 1)
 k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
             const int2 *__restrict__ tiles, int ntiles, int *ctl,
-            unsigned long long *ptime, const CUtensorMap *__restrict__ gmaps,
-            const CUtensorMap *__restrict__ xmaps, const float *in,
-            const float *in2, float *out, float *out_bf, int mode, int step,
+            unsigned long long *ptime, int nspans,
+            const CUtensorMap *__restrict__ gmaps,
+            const CUtensorMap *__restrict__ xmaps, const float *in_bf,
+            const float *in2_bf, float *out, float *out_bf, int mode, int step,
             int32_t *err) {
   using L = PanelRings<B>;
   constexpr int GS = L::GS, BS = L::BS;
@@ -292,10 +313,48 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  // This CTA's first tile: the tile list, the metadata and the tensor maps
+  // are the same for the whole factorisation, and so is G.
+  const int2 t_own = tiles[blockIdx.x];
+  const int nk_own = (meta[t_own.x].s_pad + PK - 1) / PK;
+  const int pre_g = nk_own < GS ? nk_own : GS;    // its stages loaded ahead
+  const int pre_b = nk_own < BS ? nk_own : BS;
+  auto load_g = [&](int s, const CUtensorMap *map, int kc, int row) {
+    const int k0 = kc * PK;
+    tc::mbar_expect_tx(&ct.gfull[s], G_BYTES);
+    tc::tma_load_2d(g_tile(s), map, k0, row, &ct.gfull[s]);
+    tc::tma_load_2d(g_tile(s) + G_HALF, map, k0 + PH, row, &ct.gfull[s]);
+  };
+  auto load_b = [&](int s, const CUtensorMap *xmap, int kc) {
+    tc::mbar_expect_tx(&ct.bfull[s], L::BOP_BYTES);
+    tc::tma_load_2d(b_op(s), xmap, 0, 2 * kc * 2 * B, &ct.bfull[s]);
+    tc::tma_load_2d(b_op(s) + L::BOP_HALF, xmap, 0, (2 * kc + 1) * 2 * B,
+                    &ct.bfull[s]);
+  };
+  if (warp == 0) {
+    if (tc::elect_one()) {
+      for (int kc = 0; kc < pre_g; ++kc) load_g(kc, gmaps + t_own.x, kc, t_own.y);
+      ct.gissued = pre_g;
+    }
+    __syncwarp();
+  }
   // everything below reads what the previous kernels wrote: the solver
   // state (which blocks run), the panels and the tile counter's reset
   pdl_wait();
-  if (threadIdx.x == 0) atomicMin(&ptime[1], globaltimer_ns());
+  if (warp == kBWarp) {
+    if (tc::elect_one()) {
+      for (int kc = 0; kc < pre_b; ++kc) load_b(kc, xmaps + t_own.x, kc);
+      ct.bissued = pre_b;
+    }
+    __syncwarp();
+  }
+  // this launch's span: its number is the count of the launches before it
+  unsigned long long launch = ~0ull;
+  if (threadIdx.x == 0 && nspans > 0) {
+    launch = *reinterpret_cast<volatile unsigned long long *>(ptime);
+    if (launch < (unsigned long long)nspans)
+      atomicMin(&ptime[1 + launch], globaltimer_ns());
+  }
   const uint32_t taddr = ct.tmem;
   const uint32_t aslots = taddr + L::ACC_COLS;    // A slot a at +128 a
   volatile int *abort_flag = &ct.abort;
@@ -304,36 +363,43 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
     if (lane == 0) atomicOr(err, kErrTimeout);
     ct.abort = 1;
   };
-  // the warps other than 0: the next tile index from the ring, -1 at the end
-  auto next_tile = [&](int &got, int &idx) -> bool {
-    const int q = got % kTq;
-    const bool ok = __all_sync(
-        0xffffffffu,
-        tc::mbar_wait(&ct.tfull[q], (got / kTq) & 1, kSpinP) && !*abort_flag);
-    if (!ok) {
-      give_up();
-      return false;
+  // the warps other than 0: the next tile index from the ring, -1 at the end.
+  // skip() runs when the stages loaded ahead are to be drained; false: give up
+  auto next_tile = [&](int &got, int &idx, auto skip) -> bool {
+    for (;;) {
+      const int q = got % kTq;
+      const bool ok = __all_sync(
+          0xffffffffu,
+          tc::mbar_wait(&ct.tfull[q], (got / kTq) & 1, kSpinP) && !*abort_flag);
+      if (!ok) {
+        give_up();
+        return false;
+      }
+      idx = *reinterpret_cast<volatile int *>(&ct.tq[q]);
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&ct.tempty[q]);
+      ++got;
+      if (idx != kSkip) return idx >= 0;
+      if (!skip()) {
+        give_up();
+        return false;
+      }
     }
-    idx = *reinterpret_cast<volatile int *>(&ct.tq[q]);
-    __syncwarp();
-    if (lane == 0) tc::mbar_arrive(&ct.tempty[q]);
-    ++got;
-    return idx >= 0;
   };
+  auto no_skip = [] { return true; };
 
   if (warp == 0) {
     // tiles and G stages; the whole warp runs the loop (warp-uniform
     // addresses) and one lane issues
-    int g = 0, pub = 0;
+    int g = pre_g, pub = 0;
     const int first = (int)gridDim.x;     // tiles below this: one per CTA
     for (;;) {
       int idx = -1;
       if (lane == 0) {
         // the CTA's own tile first, with no atomic; then the counter, which
         // numbers the tiles from gridDim.x on
-        if (pub == 0 && (int)blockIdx.x < ntiles &&
-            tile_active(state, tiles[blockIdx.x], mode, step)) {
-          idx = (int)blockIdx.x;
+        if (pub == 0) {
+          idx = tile_active(state, t_own, mode, step) ? (int)blockIdx.x : kSkip;
         } else {
           for (;;) {
             const int i = first + atomicAdd(&ctl[0], 1);
@@ -362,6 +428,7 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
       }
       __syncwarp();
       ++pub;
+      if (idx == kSkip) continue;
       if (idx < 0) break;
       const int2 t = tiles[idx];
       const BlockMeta bm = meta[t.x];
@@ -369,7 +436,7 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
       // s_pad is a multiple of 32: a last half stage reads zeros past s_pad
       const int nk = (bm.s_pad + PK - 1) / PK;
       const CUtensorMap *map = gmaps + t.x;
-      for (int kc = 0; kc < nk; ++kc, ++g) {
+      for (int kc = pub == 1 ? pre_g : 0; kc < nk; ++kc, ++g) {
         const int s = g % GS;
         ok = __all_sync(0xffffffffu,
                         tc::mbar_wait(&ct.gempty[s], ((g / GS) & 1) ^ 1,
@@ -379,41 +446,50 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
           break;
         }
         if (tc::elect_one()) {
-          const int k0 = kc * PK;
-          tc::mbar_expect_tx(&ct.gfull[s], G_BYTES);
-          tc::tma_load_2d(g_tile(s), map, k0, t.y, &ct.gfull[s]);
-          tc::tma_load_2d(g_tile(s) + G_HALF, map, k0 + PH, t.y, &ct.gfull[s]);
+          load_g(s, map, kc, t.y);
           ct.gissued = g + 1;
         }
         __syncwarp();
       }
       if (!ok) break;
     }
+    // the last CTA that claims no more resets the counters for the next launch
+    if (lane == 0) {
+      __threadfence();
+      if (atomicAdd(&ctl[1], 1) == (int)gridDim.x - 1) {
+        atomicExch(&ctl[0], 0);
+        atomicExch(&ctl[1], 0);
+        atomicAdd(&ptime[0], 1ull);          // launches
+      }
+    }
+    __syncwarp();
   } else if (warp == kBWarp) {
     // B stages: the B-form chunks 2 kc and 2 kc + 1 of the tile's panel
     // (past the last: zero fill)
-    int got = 0, idx = -1, gb = 0;
-    while (next_tile(got, idx)) {
+    int got = 0, idx = -1, gb = pre_b, ahead = pre_b;
+    auto skip = [&]() -> bool {
+      ahead = 0;
+      return true;
+    };
+    while (next_tile(got, idx, skip)) {
       const int2 t = tiles[idx];
       const BlockMeta bm = meta[t.x];
       const int nk = (bm.s_pad + PK - 1) / PK;
       const CUtensorMap *xmap = xmaps + t.x;
       bool ok = true;
-      for (int kc = 0; kc < nk; ++kc, ++gb) {
+      for (int kc = ahead; kc < nk; ++kc, ++gb) {
         const int s = gb % BS;
         ok = __all_sync(0xffffffffu,
                         tc::mbar_wait(&ct.bempty[s], ((gb / BS) & 1) ^ 1,
                                       kSpinP) && !*abort_flag);
         if (!ok) break;
         if (tc::elect_one()) {
-          tc::mbar_expect_tx(&ct.bfull[s], L::BOP_BYTES);
-          tc::tma_load_2d(b_op(s), xmap, 0, 2 * kc * 2 * B, &ct.bfull[s]);
-          tc::tma_load_2d(b_op(s) + L::BOP_HALF, xmap, 0,
-                          (2 * kc + 1) * 2 * B, &ct.bfull[s]);
+          load_b(s, xmap, kc);
           ct.bissued = gb + 1;
         }
         __syncwarp();
       }
+      ahead = 0;
       if (!ok) {
         give_up();
         break;
@@ -423,8 +499,21 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
     // the whole warp runs the loop (warp-uniform descriptors); one lane issues
     constexpr uint32_t idesc2 = tc::idesc_tf32_f32(PT, 2 * B);
     constexpr uint32_t idesc1 = tc::idesc_tf32_f32(PT, B);
-    int got = 0, idx = -1, gm = 0, tl = 0;
-    while (next_tile(got, idx)) {
+    // gm counts B stages, ga A slots (skipped B stages fill no slot). The
+    // skipped stages are drained here, by the warp that tests bfull: it must
+    // see each phase of a stage, as a parity test tells only odd from even.
+    int got = 0, idx = -1, gm = 0, ga = 0, tl = 0;
+    auto skip = [&]() -> bool {
+      for (; gm < pre_b; ++gm) {
+        if (!__all_sync(0xffffffffu, tc::mbar_wait(&ct.bfull[gm], 0, kSpinP)))
+          return false;
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&ct.bempty[gm]);
+      }
+      if (lane == 0) ct.bconsumed = gm;
+      return true;
+    };
+    while (next_tile(got, idx, skip)) {
       const BlockMeta bm = meta[tiles[idx].x];
       const int nk = (bm.s_pad + PK - 1) / PK;
       bool ok = true;
@@ -434,12 +523,12 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
                         tc::mbar_wait(&ct.accfree, (tl - 1) & 1, kSpinP) &&
                             !*abort_flag);
       }
-      for (int kc = 0; ok && kc < nk; ++kc, ++gm) {
-        const int s = gm % BS, a = gm % kSlots;
+      for (int kc = 0; ok && kc < nk; ++kc, ++gm, ++ga) {
+        const int s = gm % BS, a = ga % kSlots;
         ok = __all_sync(
             0xffffffffu,
             tc::mbar_wait(&ct.bfull[s], (gm / BS) & 1, kSpinP) &&
-                tc::mbar_wait(&ct.ready[a], (gm / kSlots) & 1, kSpinP) &&
+                tc::mbar_wait(&ct.ready[a], (ga / kSlots) & 1, kSpinP) &&
                 !*abort_flag);
         if (!ok) break;
         if (lane == 0) ct.bconsumed = gm + 1;
@@ -465,14 +554,14 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
         }
         __syncwarp();
       }
-      if (!ok) {
-        give_up();
-        break;
-      }
+      if (!ok) give_up();
       if (tc::elect_one()) tc::mma_commit(&ct.done);
       __syncwarp();
       ++tl;
+      if (!ok) break;
     }
+    // no MMA in flight when the CTA ends, whatever the epilogue waited for
+    if (tl > 0) tc::mbar_wait(&ct.done, (tl - 1) & 1, kSpinP);
   } else if (warp < 2 + kPConv) {
     // converters: warps 2 .. 2 + kPConv - 1. Warp w may touch TMEM lanes
     // 32 (w mod 4) .. +31, so kPConv / 4 warps share each lane quarter, one
@@ -484,14 +573,26 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
     const int kq = (warp - 2) >> 2;
     const int r = q * 32 + lane;                  // G tile row of this thread
     const uint32_t lrow = (uint32_t)(q * 32) << 16;
-    int got = 0, idx = -1, gc = 0, tl = 0;
-    while (next_tile(got, idx)) {
+    // gc counts G stages, ga A slots
+    int got = 0, idx = -1, gc = 0, ga = 0;
+    auto skip = [&]() -> bool {
+      for (int s = 0; s < pre_g; ++s) {
+        if (!__all_sync(0xffffffffu, tc::mbar_wait(&ct.gfull[s], 0, kSpinP)))
+          return false;
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&ct.gempty[s]);
+      }
+      gc = pre_g;
+      if (cid == 0) ct.gconsumed = gc;
+      return true;
+    };
+    while (next_tile(got, idx, skip)) {
       const int2 t = tiles[idx];
       const BlockMeta bm = meta[t.x];
       const int nk = (bm.s_pad + PK - 1) / PK;
       bool ok = true;
-      for (int kc = 0; kc < nk; ++kc, ++gc) {
-        const int s = gc % GS, a = gc % kSlots;
+      for (int kc = 0; kc < nk; ++kc, ++gc, ++ga) {
+        const int s = gc % GS, a = ga % kSlots;
         // warp-uniform: every lane breaks, or none does
         ok = __all_sync(0xffffffffu,
                         tc::mbar_wait(&ct.gfull[s], (gc / GS) & 1, kSpinP) &&
@@ -522,7 +623,7 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
         if (lane == 0) tc::mbar_arrive(&ct.gempty[s]);
         // the A slot's previous MMAs have completed
         ok = __all_sync(0xffffffffu,
-                        tc::mbar_wait(&ct.afree[a], ((gc / kSlots) & 1) ^ 1,
+                        tc::mbar_wait(&ct.afree[a], ((ga / kSlots) & 1) ^ 1,
                                       kSpinP) && !*abort_flag);
         if (!ok) break;
         tc::fence_after_sync();
@@ -539,7 +640,6 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
         give_up();
         break;
       }
-      ++tl;
     }
   } else {
     // the epilogue: warps 10-13, one per TMEM lane quarter (warp mod 4).
@@ -550,9 +650,57 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
     const int r = q * 32 + lane;                  // G tile row of this thread
     const uint32_t lrow = (uint32_t)(q * 32) << 16;
     int got = 0, idx = -1, tl = 0;
-    while (next_tile(got, idx)) {
+    while (next_tile(got, idx, no_skip)) {
       const int2 t = tiles[idx];
       const BlockMeta bm = meta[t.x];
+      const SolverState &st = state[t.x];
+      float alpha, beta, gamma;
+      cheb_coeffs(st, mode, step, &alpha, &beta, &gamma);
+      // the rows of `out` are read by others only after a product (mode 0)
+      // or the block's last filter step; in between, the B form is enough
+      const bool rows = mode == 0 || step == st.degree;
+      const int rr = t.y + r;                      // output row
+      const bool live = rr < bm.s_pad;
+      // B form: chunk rr / 32, position rr mod 32 (lanes of a warp hold 32
+      // consecutive rows of one chunk: coalesced 128 bytes)
+      const int64_t bo = 2 * bm.x_off + (int64_t)(rr >> 5) * 2 * B * 32 + (rr & 31);
+      const float *i1 = in_bf + bo;
+      const float *i2 = in2_bf ? in2_bf + bo : nullptr;
+      float *bfb = out_bf ? out_bf + bo : nullptr;
+      float *orow = out + bm.x_off + (int64_t)rr * B;
+      // in and in2 come from their B forms too (hi + lo is the value
+      // exactly), CH columns ahead, the first before the tile's MMAs are
+      // done: `out` may be in2, so the compiler keeps a load behind the
+      // stores before it in the program. At b = 64 the accumulators leave
+      // registers for 8 columns, and only once they have been read.
+      constexpr int CH = B <= 32 ? 16 : 8;
+      float h1[CH], l1[CH], h2[CH], l2[CH], x1[CH], x2[CH];
+      auto fetch = [&](int c0) {
+#pragma unroll
+        for (int u = 0; u < CH; ++u) {
+          const int c = c0 + u;
+          h1[u] = l1[u] = h2[u] = l2[u] = 0.f;
+          if (live && beta != 0.f) {
+            h1[u] = i1[c * 32];
+            l1[u] = i1[(B + c) * 32];
+          }
+          if (live && gamma != 0.f) {
+            h2[u] = i2[c * 32];
+            l2[u] = i2[(B + c) * 32];
+          }
+        }
+      };
+      auto join = [&]() {
+#pragma unroll
+        for (int u = 0; u < CH; ++u) {
+          x1[u] = __fadd_rn(h1[u], l1[u]);
+          x2[u] = __fadd_rn(h2[u], l2[u]);
+        }
+      };
+      if (B <= 32) {
+        fetch(0);
+        join();
+      }
       bool ok = __all_sync(0xffffffffu,
                            tc::mbar_wait(&ct.done, tl & 1, kSpinP) &&
                                !*abort_flag);
@@ -569,55 +717,46 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
         acc_sum<B>(taddr + lrow, c0, v);        // main halves
         acc_sum<B>(taddr + lrow, B + c0, w);    // cross halves
 #pragma unroll
-        for (int u = 0; u < 16; ++u) acc[c0 + u] = v[u] + w[u];
+        for (int u = 0; u < 16; ++u) acc[c0 + u] = alpha * (v[u] + w[u]);
       }
       // the accumulators may be overwritten by the next tile's MMAs
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&ct.accfree);
-      const SolverState st = state[t.x];
-      float alpha, beta, gamma;
-      cheb_coeffs(st, mode, step, &alpha, &beta, &gamma);
-      const int rr = t.y + r;                    // output row
-      if (rr < bm.s_pad) {
-        const float *inb = in + bm.x_off;
-        const float *in2b = in2 ? in2 + bm.x_off : nullptr;
-        float *outb = out + bm.x_off;
-        // B form of `out`: chunk rr / 32, position rr mod 32 (lanes of a
-        // warp hold 32 consecutive rows of one chunk: coalesced 128 bytes)
-        float *bfb = out_bf ? out_bf + 2 * bm.x_off +
-                                  (int64_t)(rr >> 5) * 2 * B * 32 + (rr & 31)
-                            : nullptr;
-        // a thread's row of `out` (and of in, in2) is contiguous: 16-byte
-        // accesses, 4 columns each
-        const int64_t o0 = (int64_t)rr * B;
+      if (B > 32) {
+        fetch(0);
+        join();
+      }
 #pragma unroll
-        for (int c4 = 0; c4 < B / 4; ++c4) {
-          float y[4];
+      for (int c0 = 0; c0 < B; c0 += CH) {
+        float v[CH];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) y[u] = alpha * acc[4 * c4 + u];
-          if (beta != 0.f) {
-            const float4 x = *reinterpret_cast<const float4 *>(inb + o0 + 4 * c4);
-            y[0] = fmaf(beta, x.x, y[0]); y[1] = fmaf(beta, x.y, y[1]);
-            y[2] = fmaf(beta, x.z, y[2]); y[3] = fmaf(beta, x.w, y[3]);
-          }
-          if (gamma != 0.f) {
-            const float4 x = *reinterpret_cast<const float4 *>(in2b + o0 + 4 * c4);
-            y[0] = fmaf(gamma, x.x, y[0]); y[1] = fmaf(gamma, x.y, y[1]);
-            y[2] = fmaf(gamma, x.z, y[2]); y[3] = fmaf(gamma, x.w, y[3]);
-          }
-          *reinterpret_cast<float4 *>(outb + o0 + 4 * c4) =
-              make_float4(y[0], y[1], y[2], y[3]);
-          if (bfb) {
+        for (int u = 0; u < CH; ++u) v[u] = acc[c0 + u];
+        if (beta != 0.f) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int c = 4 * c4 + u;
-              const float yh = hi1(y[u]);
-              bfb[c * 32] = yh;
-              bfb[(B + c) * 32] = __fsub_rn(y[u], yh);
-            }
+          for (int u = 0; u < CH; ++u) v[u] = fmaf(beta, x1[u], v[u]);
+        }
+        if (gamma != 0.f) {
+#pragma unroll
+          for (int u = 0; u < CH; ++u) v[u] = fmaf(gamma, x2[u], v[u]);
+        }
+        if (c0 + CH < B) fetch(c0 + CH);
+        if (live && rows) {
+#pragma unroll
+          for (int c4 = 0; c4 < CH / 4; ++c4)
+            *reinterpret_cast<float4 *>(orow + c0 + 4 * c4) = make_float4(
+                v[4 * c4], v[4 * c4 + 1], v[4 * c4 + 2], v[4 * c4 + 3]);
+        }
+        if (live && bfb) {
+#pragma unroll
+          for (int u = 0; u < CH; ++u) {
+            const int c = c0 + u;
+            const float yh = hi1(v[u]);
+            bfb[c * 32] = yh;
+            bfb[(B + c) * 32] = __fsub_rn(v[u], yh);
           }
         }
+        if (c0 + CH < B) join();
       }
       ++tl;
     }
@@ -635,23 +774,8 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
     for (int g = ct.bconsumed; g < ct.bissued; ++g)
       tc::mbar_wait(&ct.bfull[g % BS], (g / BS) & 1, kSpinP);
   }
-  if (threadIdx.x == 0) {
-    // the last CTA out resets the tile counter for the next launch
-    __threadfence();
-    if (atomicAdd(&ctl[1], 1) == (int)gridDim.x - 1) {
-      // and adds this launch's span (first start to last end) to ptime[0]
-      // (the two dies' timers may differ by a little: a negative span of a
-      // very short launch counts as 0)
-      const unsigned long long t0 = atomicAdd(&ptime[1], 0ull);
-      const unsigned long long t1 = globaltimer_ns();
-      if (t1 > t0 && t0 != ~0ull) atomicAdd(&ptime[0], t1 - t0);
-      atomicAdd(&ptime[2], 1ull);          // launches
-      atomicExch(&ptime[1], ~0ull);
-      atomicExch(&ctl[0], 0);
-      atomicExch(&ctl[1], 0);
-      __threadfence();
-    }
-  }
+  if (threadIdx.x == 0 && launch < (unsigned long long)nspans)
+    atomicMax(&ptime[1 + nspans + launch], globaltimer_ns());
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(taddr, kTmemCols);
 }
@@ -659,9 +783,9 @@ k_gpanel_tc(const BlockMeta *__restrict__ meta, SolverState *state,
 template <int B>
 cudaError_t launch_b(const BlockMeta *meta, SolverState *state,
                      const int2 *tiles, int32_t ntiles, int32_t nctas, int *ctl,
-                     unsigned long long *ptime,
+                     unsigned long long *ptime, int32_t nspans,
                      const CUtensorMap *gmaps, const CUtensorMap *xmaps,
-                     const float *in, const float *in2, float *out,
+                     const float *in_bf, const float *in2_bf, float *out,
                      float *out_bf, int mode, int step, int32_t *err,
                      cudaStream_t st) {
   static_assert(panel_ring_smem<B>() <= 227 * 1024, "shared memory");
@@ -673,8 +797,8 @@ cudaError_t launch_b(const BlockMeta *meta, SolverState *state,
   // of the previous kernel in the stream (see pdl_wait)
   return launch_pdl(k_gpanel_tc<B>, dim3((unsigned)nctas), dim3(kPThreads),
                     panel_ring_smem<B>(), st, meta, state, tiles, (int)ntiles,
-                    ctl, ptime, gmaps, xmaps, in, in2, out, out_bf, mode, step,
-                    err);
+                    ctl, ptime, (int)nspans, gmaps, xmaps, in_bf, in2_bf, out,
+                    out_bf, mode, step, err);
 }
 
 // F_L = W^T F_s on the tensor cores, with the panel product's data path and
@@ -969,10 +1093,10 @@ k_bform(const BlockMeta *__restrict__ meta, const SolverState *__restrict__ stat
 cudaError_t launch_gpanel_tc(int32_t bsub, const BlockMeta *meta,
                              SolverState *state, const int2 *tiles,
                              int32_t ntiles, int32_t nctas, int32_t *ctl,
-                             unsigned long long *ptime,
+                             unsigned long long *ptime, int32_t nspans,
                              const CUtensorMap *gmaps,
-                             const CUtensorMap *xmaps, const float *in,
-                             const float *in2, float *out, float *out_bf,
+                             const CUtensorMap *xmaps, const float *in_bf,
+                             const float *in2_bf, float *out, float *out_bf,
                              int mode, int step, int32_t *err,
                              cudaStream_t st) {
   if (ntiles <= 0) return cudaSuccess;
@@ -980,14 +1104,14 @@ cudaError_t launch_gpanel_tc(int32_t bsub, const BlockMeta *meta,
   if (nctas < 1) nctas = 1;
   switch (bsub) {
     case 16: return launch_b<16>(meta, state, tiles, ntiles, nctas, ctl, ptime,
-                                 gmaps, xmaps, in, in2, out, out_bf, mode, step,
-                                 err, st);
+                                 nspans, gmaps, xmaps, in_bf, in2_bf, out,
+                                 out_bf, mode, step, err, st);
     case 32: return launch_b<32>(meta, state, tiles, ntiles, nctas, ctl, ptime,
-                                 gmaps, xmaps, in, in2, out, out_bf, mode, step,
-                                 err, st);
+                                 nspans, gmaps, xmaps, in_bf, in2_bf, out,
+                                 out_bf, mode, step, err, st);
     case 64: return launch_b<64>(meta, state, tiles, ntiles, nctas, ctl, ptime,
-                                 gmaps, xmaps, in, in2, out, out_bf, mode, step,
-                                 err, st);
+                                 nspans, gmaps, xmaps, in_bf, in2_bf, out,
+                                 out_bf, mode, step, err, st);
     default: return cudaErrorInvalidValue;
   }
 }
