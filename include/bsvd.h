@@ -183,6 +183,20 @@ bsvd_status bsvd_partition_diag(bsvd_ctx *ctx, int32_t nb,
                                 const float *x);
 
 /*
+ * bsvd_partition_diag from each matrix's own arrays: piece b of u holds
+ * nu[b] row ids of matrix b in its own coordinates (0 .. m_b - 1), piece b
+ * of i and x its columns and ratings (host or device memory, read before the
+ * call returns). The pieces are put one after the other on the device, so
+ * the caller builds no stacked copy; sum(nu) = sum(ni) = sum(nx).
+ */
+bsvd_status bsvd_partition_batch(bsvd_ctx *ctx, int32_t nb,
+                                 const int64_t *row_bounds,
+                                 const int64_t *col_bounds,
+                                 const int32_t *const *u, const int64_t *nu,
+                                 const int32_t *const *i, const int64_t *ni,
+                                 const float *const *x, const int64_t *nx);
+
+/*
  * Uneven grid cut at rating-activity quantiles, for bsvd_partition (the
  * batched form; the paper's own grid, Section 3 Eq. "datax", has equal
  * blocks, which on long-tailed data leaves a few blocks holding most

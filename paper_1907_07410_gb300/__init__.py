@@ -31,7 +31,7 @@ EXPORTS = ("bsvd_config_default", "bsvd_create", "bsvd_destroy",
            "bsvd_rmse", "bsvd_block_stats", "bsvd_get_block",
            "bsvd_reconstruct", "bsvd_factor_report", "bsvd_phase_times",
            "bsvd_kernel_launches", "bsvd_block_means_noalloc",
-           "bsvd_gram_path", "bsvd_partition_diag", "bsvd_factor_ks",
+           "bsvd_gram_path", "bsvd_partition_diag", "bsvd_partition_batch", "bsvd_factor_ks",
            "bsvd_sgd_params_default", "bsvd_sgd_prepare", "bsvd_sgd_train",
            "bsvd_sgd_predict", "bsvd_sgd_get", "bsvd_quantile_grid",
            "bsvd_partition_quantile",
@@ -92,6 +92,7 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
                                  vp, vp, vp]),
         "bsvd_factor": (i32, [vp, i32]),
         "bsvd_partition_diag": (i32, [vp, i32, vp, vp, i64, vp, vp, vp]),
+        "bsvd_partition_batch": (i32, [vp, i32] + [vp] * 8),
         "bsvd_factor_ks": (i32, [vp, vp]),
         "bsvd_predict": (i32, [vp, i64, vp, vp, vp]),
         "bsvd_rmse": (i32, [vp, i64, vp, vp, vp, ctypes.POINTER(ctypes.c_double)]),
@@ -262,6 +263,32 @@ def bsvd_partition_diag(ctx, row_bounds, col_bounds, u, i, x) -> int:
         ctx, rb.size - 1, rb.ctypes.data, cb.ctypes.data, nnz,
         _ptr(u, np.int32, "u"), _ptr(i, np.int32, "i"),
         _ptr(x, np.float32, "x"))
+    return _check(ctx, st)
+
+
+def bsvd_partition_batch(ctx, row_bounds, col_bounds, us, is_, xs) -> int:
+    """us, is_, xs: one array per matrix, ids in the matrix's own
+    coordinates."""
+    rb = np.ascontiguousarray(row_bounds, np.int64)
+    cb = np.ascontiguousarray(col_bounds, np.int64)
+    nb = rb.size - 1
+    if rb.size != cb.size or nb < 1:
+        raise ValueError("row_bounds and col_bounds need nb + 1 entries")
+    args, total = [], []
+    for pieces, dtype, name in ((us, np.int32, "u"), (is_, np.int32, "i"),
+                                (xs, np.float32, "x")):
+        if len(pieces) != nb:
+            raise ValueError("%s needs one piece per matrix" % name)
+        lens = np.array([_len(a) for a in pieces], np.int64)
+        args += [(ctypes.c_void_p * nb)(*[_ptr(a, dtype, name)
+                                          for a in pieces]), lens]
+        total.append(int(lens.sum()))
+    if total[1] != total[0] or total[2] != total[0]:
+        raise ValueError("u, i, x must have the same length")
+    st = load().bsvd_partition_batch(
+        ctx, nb, rb.ctypes.data, cb.ctypes.data,
+        *[a.ctypes.data if isinstance(a, np.ndarray) else ctypes.addressof(a)
+          for a in args])
     return _check(ctx, st)
 
 
@@ -573,6 +600,11 @@ class Context:
 
     def partition_diag(self, row_bounds, col_bounds, u, i, x):
         bsvd_partition_diag(self.handle, row_bounds, col_bounds, u, i, x)
+        self.nblocks = len(row_bounds) - 1
+
+    def partition_batch(self, row_bounds, col_bounds, us, is_, xs):
+        """partition_diag from one array of each kind per matrix."""
+        bsvd_partition_batch(self.handle, row_bounds, col_bounds, us, is_, xs)
         self.nblocks = len(row_bounds) - 1
 
     def factor(self, k, warn=True):

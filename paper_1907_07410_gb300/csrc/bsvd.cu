@@ -124,6 +124,9 @@ struct bsvd_ctx {
   DevBuf d_lpart, d_spart, d_flip;
   // the persistent panel products' tile counter, and the CTAs they launch
   DevBuf d_pctl;
+  // the pieces of bsvd_partition_batch: where each begins in the stacked ids
+  DevBuf d_pieces;
+  std::vector<int64_t> h_pieces;
   int32_t nsm = 1;
   // panel products: [0] launches, then (profile = 1) the starts and the ends
   // of the first nspans of them; the graph loop's step counter
@@ -585,7 +588,7 @@ void bsvd_destroy(bsvd_ctx *c) {
                     &c->d_qperm2,
                     &c->d_qbounds, &c->d_pbmaps, &c->d_fbmaps, &c->d_FB,
                     &c->d_lpart, &c->d_spart, &c->d_flip, &c->d_pctl,
-                    &c->d_ptime, &c->d_loopctl, &c->d_finv, &c->d_chunks};
+                    &c->d_ptime, &c->d_pieces, &c->d_loopctl, &c->d_finv, &c->d_chunks};
   if (c->st) cudaStreamSynchronize(c->st);
   else cudaDeviceSynchronize();
   if (c->up) cudaStreamSynchronize(c->up);
@@ -607,13 +610,24 @@ const char *bsvd_last_error(const bsvd_ctx *c) {
   return c ? c->err.c_str() : "null context";
 }
 
+// The rating arrays of bsvd_partition_batch: one piece of each per matrix.
+struct Pieces {
+  const int32_t *const *u;
+  const int64_t *nu;
+  const int32_t *const *i;
+  const int64_t *ni;
+  const float *const *x;
+  const int64_t *nx;
+};
+
 static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
                                   int64_t nnz, const int32_t *u,
                                   const int32_t *i, const float *x, int32_t p,
                                   int32_t q, const int64_t *row_bounds,
                                   const int64_t *col_bounds,
                                   const int32_t *row_perm,
-                                  const int32_t *col_perm, bool diag) {
+                                  const int32_t *col_perm, bool diag,
+                                  const Pieces *pieces = nullptr) {
   if (!c) return BSVD_EINVAL;
   c->err.clear();
   c->sgd_ready = false;      // a new grid invalidates the SGD order
@@ -623,7 +637,7 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
                 (long long)m, (long long)n, (long long)nnz);
   if (p < 1 || q < 1 || (!row_bounds && p > m) || (!col_bounds && q > n))
     return fail(c, BSVD_EINVAL, "partition: bad grid %d x %d", p, q);
-  if (nnz > 0 && (!u || !i || !x))
+  if (nnz > 0 && !pieces && (!u || !i || !x))
     return fail(c, BSVD_EINVAL, "partition: null rating arrays");
   if ((int64_t)p * q > (int64_t)INT32_MAX)
     return fail(c, BSVD_EINVAL, "partition: too many blocks");
@@ -730,9 +744,44 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
   }
 
   const void *du = nullptr, *di = nullptr, *dx = nullptr;
-  CK(device_view(c, u, sizeof(int32_t) * nnz, c->s_a, &du), "partition");
-  CK(device_view(c, i, sizeof(int32_t) * nnz, c->s_b, &di), "partition");
-  CK(device_view(c, x, sizeof(float) * nnz, c->s_c, &dx), "partition");
+  if (pieces) {
+    // each piece goes to its place in the staging buffers; then the ids are
+    // moved to the stacked coordinates there
+    c->h_pieces.assign(2 * (size_t)(nb + 1), 0);
+    auto gather = [&](const void *src, const int64_t *len, int64_t *starts,
+                      DevBuf &stage, const void **out) -> cudaError_t {
+      cudaError_t e = stage.ensure(4 * std::max<int64_t>(nnz, 1));
+      const void *const *from = static_cast<const void *const *>(src);
+      int64_t at = 0;
+      for (int32_t b = 0; b < nb && e == cudaSuccess; ++b) {
+        if (starts) starts[b] = at;
+        if (len[b] > 0)
+          e = cudaMemcpyAsync(stage.as<char>() + 4 * at, from[b], 4 * len[b],
+                              cudaMemcpyDefault, c->st);
+        at += len[b];
+      }
+      if (starts) starts[nb] = at;
+      *out = stage.p;
+      return e;
+    };
+    int64_t *su = c->h_pieces.data(), *si = su + nb + 1;
+    CK(gather(pieces->u, pieces->nu, su, c->s_a, &du), "partition");
+    CK(gather(pieces->i, pieces->ni, si, c->s_b, &di), "partition");
+    CK(gather(pieces->x, pieces->nx, nullptr, c->s_c, &dx), "partition");
+    CK(c->d_pieces.ensure(sizeof(int64_t) * c->h_pieces.size()), "partition");
+    CK(cudaMemcpyAsync(c->d_pieces.p, su, sizeof(int64_t) * c->h_pieces.size(),
+                       cudaMemcpyHostToDevice, c->st), "partition");
+    const int64_t *ds = c->d_pieces.as<int64_t>();
+    CK(launch_stack_ids(nnz, nb, ds, c->d_rb.as<int64_t>(),
+                        c->s_a.as<int32_t>(), c->st), "partition");
+    CK(launch_stack_ids(nnz, nb, ds + nb + 1, c->d_cb.as<int64_t>(),
+                        c->s_b.as<int32_t>(), c->st), "partition");
+    c->launches += nnz > 0 ? 2 : 0;
+  } else {
+    CK(device_view(c, u, sizeof(int32_t) * nnz, c->s_a, &du), "partition");
+    CK(device_view(c, i, sizeof(int32_t) * nnz, c->s_b, &di), "partition");
+    CK(device_view(c, x, sizeof(float) * nnz, c->s_c, &dx), "partition");
+  }
 
   CK(cudaMemsetAsync(c->d_counts.p, 0, sizeof(unsigned long long) * nb, c->st),
      "partition");
@@ -897,6 +946,36 @@ bsvd_status bsvd_partition_diag(bsvd_ctx *c, int32_t nb,
     return fail(c, BSVD_EINVAL, "partition_diag: need nb >= 1 and bounds");
   return partition_impl(c, row_bounds[nb], col_bounds[nb], nnz, u, i, x, nb,
                         nb, row_bounds, col_bounds, nullptr, nullptr, true);
+}
+
+bsvd_status bsvd_partition_batch(bsvd_ctx *c, int32_t nb,
+                                 const int64_t *row_bounds,
+                                 const int64_t *col_bounds,
+                                 const int32_t *const *u, const int64_t *nu,
+                                 const int32_t *const *i, const int64_t *ni,
+                                 const float *const *x, const int64_t *nx) {
+  if (!c) return BSVD_EINVAL;
+  c->err.clear();
+  if (nb < 1 || !row_bounds || !col_bounds)
+    return fail(c, BSVD_EINVAL, "partition_batch: need nb >= 1 and bounds");
+  if (!u || !nu || !i || !ni || !x || !nx)
+    return fail(c, BSVD_EINVAL, "partition_batch: null piece arrays");
+  int64_t tu = 0, ti = 0, tx = 0;
+  for (int32_t b = 0; b < nb; ++b) {
+    if (nu[b] < 0 || ni[b] < 0 || nx[b] < 0 || (nu[b] && !u[b]) ||
+        (ni[b] && !i[b]) || (nx[b] && !x[b]))
+      return fail(c, BSVD_EINVAL, "partition_batch: bad pieces of matrix %d", b);
+    tu += nu[b];
+    ti += ni[b];
+    tx += nx[b];
+  }
+  if (tu != ti || tu != tx)
+    return fail(c, BSVD_EINVAL, "partition_batch: %lld rows, %lld columns and "
+                "%lld ratings", (long long)tu, (long long)ti, (long long)tx);
+  const Pieces pieces = {u, nu, i, ni, x, nx};
+  return partition_impl(c, row_bounds[nb], col_bounds[nb], tu, nullptr,
+                        nullptr, nullptr, nb, nb, row_bounds, col_bounds,
+                        nullptr, nullptr, true, &pieces);
 }
 
 // One side of the activity-quantile grid: perm (host or device, size
