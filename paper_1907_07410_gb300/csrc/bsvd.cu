@@ -126,6 +126,7 @@ struct bsvd_ctx {
   DevBuf d_pctl;
   // the pieces of bsvd_partition_batch: where each begins in the stacked ids
   DevBuf d_pieces;
+  DevBuf d_pchunks;          // ratings per plane chunk, then their lists' ends
   std::vector<int64_t> h_pieces;
   int32_t nsm = 1;
   // panel products: [0] launches, then (profile = 1) the starts and the ends
@@ -588,7 +589,7 @@ void bsvd_destroy(bsvd_ctx *c) {
                     &c->d_qperm2,
                     &c->d_qbounds, &c->d_pbmaps, &c->d_fbmaps, &c->d_FB,
                     &c->d_lpart, &c->d_spart, &c->d_flip, &c->d_pctl,
-                    &c->d_ptime, &c->d_pieces, &c->d_loopctl, &c->d_finv, &c->d_chunks};
+                    &c->d_ptime, &c->d_pieces, &c->d_pchunks, &c->d_loopctl, &c->d_finv, &c->d_chunks};
   if (c->st) cudaStreamSynchronize(c->st);
   else cudaDeviceSynchronize();
   if (c->up) cudaStreamSynchronize(c->up);
@@ -668,7 +669,7 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
 
   // block shapes and the dense arena layout
   c->meta.assign(c->nblocks, BlockMeta());
-  int64_t off = 0, vxoff = 0;
+  int64_t off = 0, vxoff = 0, nchunks = 0;
   for (int32_t bi = 0; bi < p; ++bi) {
     for (int32_t bj = 0; bj < q; ++bj) {
       if (diag && bi != bj) continue;
@@ -688,11 +689,15 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
       bm.w_off = off;
       bm.s128 = (int32_t)round_up(bm.s, 128);
       bm.vx_off = vxoff;
+      bm.ck0 = (int32_t)nchunks;
       if (!bm.owned) continue;   // another shard's block: no dense storage
       off += (int64_t)bm.s_pad * bm.L_pad;
       // exact Gram: planes [Y; M]; bf16 Gram: one bf16 copy of W
       vxoff += (c->cfg.precision == BSVD_BF16 ? 1 : 2) * (int64_t)bm.s128 *
                bm.L_pad;
+      bm.nck = (int32_t)(((int64_t)bm.s128 * bm.L_pad + kPlaneChunk - 1) /
+                         kPlaneChunk);
+      nchunks += bm.nck;
     }
   }
   c->arena = off;
@@ -790,6 +795,26 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
   CK(cudaMemsetAsync(c->d_maxabs.p, 0, sizeof(unsigned int), c->st),
      "partition");
   const GridDesc g = c->grid();
+  // Large planes are filled chunk by chunk; the lists on the way take the
+  // place of the float32 arena, which such a partition does not hold (or
+  // writes later, from the ratings)
+  const bool planes = c->tc_planes || c->cfg.precision == BSVD_BF16;
+  const bool chunked =
+      planes && !c->w32 && chunked_planes(g, nnz, nchunks, 2 * vxoff, off / 3);
+  unsigned *chunks = nullptr;
+  uint2 *where = nullptr;
+  uint32_t *list = nullptr;
+  if (chunked) {
+    CK(c->d_W.ensure(3 * sizeof(uint32_t) * nnz), "partition");
+    where = c->d_W.as<uint2>();
+    list = c->d_W.as<uint32_t>() + 2 * nnz;
+    CK(c->d_pchunks.ensure(sizeof(unsigned) * chunk_words(nchunks)),
+       "partition");
+    chunks = c->d_pchunks.as<unsigned>();
+    CK(cudaMemsetAsync(chunks, 0, sizeof(unsigned) * chunk_slots(nchunks),
+                       c->st),
+       "partition");
+  }
   auto write_w = [&]() -> bsvd_status {
     CK(c->d_W.ensure(sizeof(float) * std::max<int64_t>(off, 1)), "partition");
     CK(cudaMemsetAsync(c->d_W.p, 0, sizeof(float) * std::max<int64_t>(off, 1),
@@ -806,7 +831,8 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
   CK(launch_count(g, nnz, (const int32_t *)du, (const int32_t *)di,
                   (const float *)dx, nb, c->d_counts.as<unsigned long long>(),
                   c->d_sums.as<long long>(), c->d_maxabs.as<unsigned int>(),
-                  c->d_err.as<int32_t>(), c->st), "partition: count");
+                  c->d_err.as<int32_t>(), c->st, c->d_meta.as<BlockMeta>(),
+                  chunks, nchunks, where), "partition: count");
   CK(launch_means(nb, c->d_counts.as<unsigned long long>(),
                   c->d_sums.as<long long>(), c->d_maxabs.as<unsigned int>(),
                   c->d_mu.as<float>(), c->d_err.as<int32_t>(), c->st),
@@ -816,34 +842,43 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
     const bsvd_status ws = write_w();
     if (ws != BSVD_OK) return ws;
   }
-  if (c->cfg.precision == BSVD_BF16) {
-    CK(c->d_VX.ensure(2 * std::max<int64_t>(vxoff, 1)), "partition");
+  if (planes) CK(c->d_VX.ensure(2 * std::max<int64_t>(vxoff, 1)), "partition");
+  if (planes && !chunked)
     CK(cudaMemsetAsync(c->d_VX.p, 0, 2 * std::max<int64_t>(vxoff, 1), c->st),
        "partition");
-    CK(launch_scatter_bf16(g, c->d_meta.as<BlockMeta>(), nnz,
-                           (const int32_t *)du, (const int32_t *)di,
-                           (const float *)dx, c->d_mu.as<float>(),
-                           c->d_VX.as<__nv_bfloat16>(), c->st),
+  if (c->cfg.precision == BSVD_BF16) {
+    CK(chunked
+           ? launch_chunked_bf16(g, c->d_meta.as<BlockMeta>(), nnz, where,
+                                 (const float *)dx, c->d_mu.as<float>(),
+                                 (int32_t)nchunks, chunks, list,
+                                 c->d_VX.as<__nv_bfloat16>(), c->st)
+           : launch_scatter_bf16(g, c->d_meta.as<BlockMeta>(), nnz,
+                                 (const int32_t *)du, (const int32_t *)di,
+                                 (const float *)dx, c->d_mu.as<float>(),
+                                 c->d_VX.as<__nv_bfloat16>(), c->st),
        "partition: scatter");
-    c->launches += nnz > 0;
+    c->launches += chunked ? 4 : nnz > 0;
   }
   // bf16 planes for the exact tensor-core Gram
   c->tc_exact = false;
   if (c->tc_planes) {
-    CK(c->d_VX.ensure(2 * std::max<int64_t>(vxoff, 1)), "partition");
     CK(c->d_shift.ensure(sizeof(float) * nb), "partition");
     CK(c->d_delta.ensure(sizeof(float) * nb), "partition");
-    CK(cudaMemsetAsync(c->d_VX.p, 0, 2 * std::max<int64_t>(vxoff, 1), c->st),
-       "partition");
     CK(launch_plane_shift(nb, c->d_counts.as<unsigned long long>(),
                           c->d_sums.as<long long>(), c->d_shift.as<float>(),
                           c->d_delta.as<float>(), c->st), "partition: shift");
-    CK(launch_scatter_planes(g, c->d_meta.as<BlockMeta>(), nnz,
-                             (const int32_t *)du, (const int32_t *)di,
-                             (const float *)dx, c->d_shift.as<float>(),
-                             c->d_VX.as<__nv_bfloat16>(), c->d_err.as<int32_t>() + 1,
-                             c->st), "partition: planes");
-    c->launches += nnz > 0 ? 2 : 1;
+    int32_t *found = c->d_err.as<int32_t>() + 1;
+    CK(chunked
+           ? launch_chunked_planes(g, c->d_meta.as<BlockMeta>(), nnz, where,
+                                   (const float *)dx, c->d_shift.as<float>(),
+                                   (int32_t)nchunks, chunks, list,
+                                   c->d_VX.as<__nv_bfloat16>(), found, c->st)
+           : launch_scatter_planes(g, c->d_meta.as<BlockMeta>(), nnz,
+                                   (const int32_t *)du, (const int32_t *)di,
+                                   (const float *)dx, c->d_shift.as<float>(),
+                                   c->d_VX.as<__nv_bfloat16>(), found, c->st),
+       "partition: planes");
+    c->launches += chunked ? 5 : nnz > 0 ? 2 : 1;
   }
   mark(c, 1);
   int32_t flag = 0;

@@ -88,7 +88,12 @@ struct BlockMeta {
   int32_t pt0, npt;     // the block's 128-row tiles of F_s (panel tiles)
   int32_t pj0, npj;     // the block's 128-row tiles of F_L (projection)
   int32_t ch0, nch;     // the block's kChunkRows-row chunks (small Grams)
+  int32_t ck0, nck;     // the kPlaneChunk-cell chunks of each of its planes
 };
+
+// cells of a bf16 plane that the partition fills in shared memory at once
+constexpr int kPlaneChunkLog = 13;
+constexpr int kPlaneChunk = 1 << kPlaneChunkLog;
 
 // rows of the panels per chunk of the Rayleigh-Ritz small Grams
 constexpr int kChunkRows = 512;

@@ -19,7 +19,9 @@ cudaError_t launch_count(const GridDesc &g, int64_t nnz, const int32_t *u,
                          const int32_t *i, const float *x, int32_t nblocks,
                          unsigned long long *counts, long long *sums,
                          unsigned int *maxabs_bits, int32_t *err,
-                         cudaStream_t st);
+                         cudaStream_t st, const BlockMeta *meta = nullptr,
+                         unsigned *chunks = nullptr, int64_t nchunks = 0,
+                         uint2 *where = nullptr);
 cudaError_t launch_means(int32_t nblocks, const unsigned long long *counts,
                          const long long *sums,
                          const unsigned int *maxabs_bits, float *mu,
@@ -35,6 +37,27 @@ cudaError_t launch_scatter_bf16(const GridDesc &g, const BlockMeta *meta,
                                 const int32_t *i, const float *x,
                                 const float *mu, __nv_bfloat16 *Wh,
                                 cudaStream_t st);
+
+// The bf16 planes of a large matrix, every cell of them, chunk by chunk
+// (BlockMeta::ck0). chunks: chunk_words(nchunks) words, the first
+// chunk_slots(nchunks) the ratings per chunk from launch_count (zero before);
+// where: nnz places, from launch_count; list: nnz words.
+bool chunked_planes(const GridDesc &g, int64_t nnz, int64_t nchunks,
+                    int64_t plane_bytes, int64_t list_cap);
+int64_t chunk_slots(int64_t nchunks);
+int64_t chunk_words(int64_t nchunks);
+cudaError_t launch_chunked_bf16(const GridDesc &g, const BlockMeta *meta,
+                                int64_t nnz, const uint2 *where,
+                                const float *x, const float *mu,
+                                int32_t nchunks, unsigned *chunks,
+                                uint32_t *list, __nv_bfloat16 *Wh,
+                                cudaStream_t st);
+cudaError_t launch_chunked_planes(const GridDesc &g, const BlockMeta *meta,
+                                  int64_t nnz, const uint2 *where,
+                                  const float *x, const float *shift,
+                                  int32_t nchunks, unsigned *chunks,
+                                  uint32_t *list, __nv_bfloat16 *VX,
+                                  int32_t *flag, cudaStream_t st);
 
 // ---- activity-quantile cut of one side (kernels_grid.cu) ----------------
 // Keys are padded to quantile_cut_padded(size) entries. counts: size,

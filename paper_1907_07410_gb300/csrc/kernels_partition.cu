@@ -27,6 +27,9 @@ namespace {
 
 constexpr int kSmemBlocks = 2048;   // per-CTA histogram size limit
 constexpr int kRatings = 4;            // ratings a thread has in flight
+// planes from this size on are filled chunk by chunk (k_fill): smaller ones
+// stay in the L2 from the memset to the scatter
+constexpr int64_t kChunkedBytes = 256 << 20;
 
 // A batch's ids to the stacked coordinates, in place: 16 bytes of traffic a
 // rating; the piece is found by bisection (the table stays in the L1).
@@ -66,10 +69,19 @@ __device__ __forceinline__ bool rating_ok(float x) {
   return isfinite(x) && fabsf(x) < 2147483648.0f;
 }
 
+// x * 2^32, rounded to the nearest integer, for |x| < 2^31. From 2^-9 on it is
+// the mantissa shifted left, in integers: the product in float64 (below 2^-9)
+// is three instructions of a pipe that takes 19 cycles an SM for each, which
+// was most of k_count (10.8 million ratings: 113 -> 72 us). An integer form with a branch per exponent
+// range had been slower still.
 __device__ __forceinline__ long long fixed32(float x) {
-  // x * 2^32 is exact in float64; round to the nearest integer. (An
-  // integer-only version with a branch per exponent range measured about
-  // 1 ms slower per pass over the large workload's 90 million ratings.)
+  const uint32_t bits = __float_as_uint(x);
+  const int sh = (int)(bits >> 23 & 0xff) - 118;    // 2^-9 has exponent 118
+  if (sh >= 0) {
+    const long long v = (long long)(bits & 0x7fffffu | 0x800000u) << (sh & 63);
+    return (int32_t)bits < 0 ? -v : v;
+  }
+  if (x == 0.f) return 0;
   return __double2ll_rn(__dmul_rn((double)x, 4294967296.0));
 }
 
@@ -84,14 +96,69 @@ struct CountTable {
   BoundsTable bounds;
 };
 
-template <bool TABLE>
+// Where a cell of a block's bf16 plane is: its chunk and its place in it.
+struct Place {
+  int32_t row0, col0, L_pad, flags, ck0;   // flags as Dest
+};
+__device__ __forceinline__ Place place_of(const BlockMeta &bm) {
+  return {(int32_t)bm.row0, (int32_t)bm.col0, bm.L_pad,
+          (bm.trans ? 1 : 0) | (bm.owned ? 2 : 0), bm.ck0};
+}
+__device__ __forceinline__ int64_t plane_cell(const Place &p, int32_t ru,
+                                              int32_t ci) {
+  const int32_t r = ru - p.row0, c = ci - p.col0;
+  return (p.flags & 1) ? (int64_t)c * p.L_pad + r : (int64_t)r * p.L_pad + c;
+}
+
+// Chunk ck's counter. Neighbouring chunks are busy together (the head of a
+// long-tailed matrix is dense), and the L2 adds to one line at about one a
+// nanosecond: consecutive chunks are spread over the table, a power of two
+// long (mask + 1), which also is the order of the chunks' lists. With
+// neighbours side by side the 10.8 million additions below took 600 us.
+__device__ __forceinline__ int32_t chunk_slot(int32_t ck, uint32_t mask) {
+  return (int32_t)((uint32_t)ck * 0x9E3779B1u & mask);     // odd: one to one
+}
+
+// A rating's place in the planes: its chunk's slot, and its block and cell in
+// the chunk (16 bits each; at most kTableBlocks blocks). It is written by
+// k_count and read by k_bucket, which saves looking up the ids' positions, a
+// random access each, again.
+constexpr uint32_t kNowhere = 0xffffffffu;
+
+// One more entry in chunk ck for every lane with `on`; returns the lane's
+// place among the chunk's entries. A whole warp: when its ratings are all in
+// one chunk (a matrix sorted by rows), one lane adds for all.
+__device__ __forceinline__ unsigned chunk_add(unsigned *cnt, bool on,
+                                              int32_t ck) {
+  const unsigned m = __ballot_sync(0xffffffffu, on);
+  if (m == 0) return 0;
+  const int lane = threadIdx.x & 31, first = __ffs(m) - 1;
+  const int32_t c0 = __shfl_sync(0xffffffffu, ck, first);
+  if (__all_sync(0xffffffffu, !on || ck == c0)) {
+    unsigned base = 0;
+    if (lane == first) base = atomicAdd(&cnt[c0], (unsigned)__popc(m));
+    base = __shfl_sync(0xffffffffu, base, first);
+    return base + __popc(m & ((1u << lane) - 1));
+  }
+  return on ? atomicAdd(&cnt[ck], 1u) : 0;
+}
+
+// CHUNKS: also the ratings per plane chunk (see k_fill); then TABLE.
+template <bool TABLE, bool CHUNKS>
 __global__ void __launch_bounds__(256)
 k_count(GridDesc g, int64_t nnz, const int32_t *__restrict__ u,
         const int32_t *__restrict__ it, const float *__restrict__ x,
         int32_t nblocks, unsigned long long *counts, long long *sums,
-        unsigned int *maxabs_bits, int32_t *err) {
+        unsigned int *maxabs_bits, int32_t *err,
+        const BlockMeta *__restrict__ meta, unsigned *chunks, uint32_t mask,
+        uint2 *__restrict__ where) {
   extern __shared__ unsigned char smem[];
   CountTable &t = *reinterpret_cast<CountTable *>(smem);
+  Place *place = reinterpret_cast<Place *>(smem + sizeof(CountTable));
+  if (CHUNKS) {
+    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
+      place[b] = place_of(meta[b]);
+  }
   __shared__ unsigned int s_max;
   const bool use_smem = nblocks <= kSmemBlocks;
   if (use_smem) {
@@ -121,15 +188,30 @@ k_count(GridDesc g, int64_t nnz, const int32_t *__restrict__ u,
 #pragma unroll
     for (int k = 0; k < kRatings; ++k) {
       bool ok = t0 + k * stride + lane < nnz;
-      int32_t blk = -1, ru, ci;
+      int32_t blk = -1, ru = 0, ci = 0;
       if (ok) {
         if (!find_block<TABLE>(g, t.bounds, uu[k], ii[k], &blk, &ru, &ci)) {
           local_err |= kErrIndex;
           ok = false;
-        } else if (!rating_ok(xx[k])) {
-          local_err |= kErrValue;
-          ok = false;
         }
+      }
+      if (CHUNKS) {
+        Place pl = {};
+        if (ok) pl = place[blk];
+        const bool held = ok && (pl.flags & 2);
+        const int64_t cell = plane_cell(pl, ru, ci);
+        const int32_t slot =
+            chunk_slot(pl.ck0 + (int32_t)(cell >> kPlaneChunkLog), mask);
+        chunk_add(chunks, held, slot);
+        const int64_t e = t0 + k * stride + lane;
+        if (e < nnz)
+          where[e] = make_uint2(
+              held ? (uint32_t)slot : kNowhere,
+              (uint32_t)blk << 16 | (uint32_t)(cell & (kPlaneChunk - 1)));
+      }
+      if (ok && !rating_ok(xx[k])) {
+        local_err |= kErrValue;
+        ok = false;
       }
       const unsigned on = __ballot_sync(0xffffffffu, ok);
       if (on == 0) continue;
@@ -274,6 +356,17 @@ __device__ __forceinline__ Dest dest_of(const BlockMeta *meta,
   return d;
 }
 
+// Why y, the offset of x from sub, does not do in the planes.
+__device__ __forceinline__ int32_t plane_flags(float y, float sub, float lim,
+                                               float x) {
+  const float ay = fabsf(y);
+  int32_t bad = 0;
+  if (!(y == rintf(y) && ay <= lim)) bad |= kErrNotExact;
+  if (!(2.f * y == rintf(2.f * y) && 2.f * ay <= lim)) bad |= kErrNotHalf;
+  if (!(__fadd_rn(y, sub) == x)) bad |= kErrNotRebuilt;
+  return bad;
+}
+
 // out (zeroed): cell = x - sub, where sub is the block's mean (kToFloat,
 // kToBf16) or its rounded mean (kToPlanes: the offset y in bf16, and 1 in the
 // mask's plane). *flag (kToPlanes): kErrNotExact when some y is not a whole
@@ -329,11 +422,7 @@ k_scatter(GridDesc g, const BlockMeta *__restrict__ meta, int64_t nnz,
         o[cell] = __float2bfloat16_rn(y);
         if (TO == kToPlanes) {
           o[cell + d.mask] = __float2bfloat16_rn(1.f);
-          const float ay = fabsf(y);
-          if (!(y == rintf(y) && ay <= d.lim)) bad |= kErrNotExact;
-          if (!(2.f * y == rintf(2.f * y) && 2.f * ay <= d.lim))
-            bad |= kErrNotHalf;
-          if (!(__fadd_rn(y, d.sub) == xx[k])) bad |= kErrNotRebuilt;
+          bad |= plane_flags(y, d.sub, d.lim, xx[k]);
         }
       }
     }
@@ -342,6 +431,222 @@ k_scatter(GridDesc g, const BlockMeta *__restrict__ meta, int64_t nnz,
     const int32_t all = __reduce_or_sync(0xffffffffu, bad);
     if (all && (threadIdx.x & 31) == 0) atomicOr(flag, all);
   }
+}
+
+// The planes of a large matrix, chunk by chunk. Ratings scattered into zeroed
+// planes cost a 32-byte DRAM sector each, written part by part at 25 to 30
+// billion a second whatever the order of issue: 10.8 million ratings in
+// 3.8 GB of planes took 635 us after a memset of 590. Instead the ratings are
+// counted by chunk of 2^14 cells (in k_count), put into their chunk's list
+// (k_bucket, 4 bytes each: 14 bits of place, the bf16 offset), and a CTA lays
+// out one chunk at a time in shared memory and stores it as it is (k_fill),
+// zeros included: 157 + 667 us and 60 more in k_count; 17 GB of one plane and
+// 90 million ratings 1.5 + 3.0 ms and 0.3, from 2.7 + 3.8; 0.35 GB and 6.2
+// million in a batch 116 + 71 and 42 us, from 348 + 60. Chunks of 2^12 or 2^14
+// cells are within 5 % on the large ones; 2^14 costs the batch 60 us (fewer
+// counters, more waiting at each).
+//
+// Exclusive scan of the chunks' counts in two levels: within kScanTile
+// counts here, the tiles' totals in k_chunk_tops.
+constexpr int kScanTile = 4096;
+
+__device__ __forceinline__ unsigned scan_1024(unsigned v, unsigned *warp_sum,
+                                              unsigned *total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  unsigned inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned up = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += up;
+  }
+  if (lane == 31) warp_sum[w] = inc;
+  __syncthreads();
+  if (w == 0) {
+    const unsigned ws = warp_sum[lane];
+    unsigned wi = ws;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned up = __shfl_up_sync(0xffffffffu, wi, o);
+      if (lane >= o) wi += up;
+    }
+    warp_sum[lane] = wi - ws;
+    if (lane == 31) *total = wi;
+  }
+  __syncthreads();
+  return warp_sum[w] + inc - v;
+}
+
+__global__ void __launch_bounds__(1024)
+k_chunk_scan(int32_t nslots, unsigned *cnt, unsigned *tops) {
+  __shared__ unsigned ws[32], total;
+  const int64_t e0 = (int64_t)blockIdx.x * kScanTile + 4 * threadIdx.x;
+  unsigned v[4], sum = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = e0 + k < nslots ? cnt[e0 + k] : 0;
+    sum += v[k];
+  }
+  unsigned at = scan_1024(sum, ws, &total);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (e0 + k < nslots) cnt[e0 + k] = at;
+    at += v[k];
+  }
+  if (threadIdx.x == 0) tops[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(1024)
+k_chunk_tops(int32_t ntiles, unsigned *tops) {
+  __shared__ unsigned ws[32], total;
+  unsigned carry = 0;
+  for (int t0 = 0; t0 < ntiles; t0 += 1024) {
+    const int t = t0 + threadIdx.x;
+    const unsigned v = t < ntiles ? tops[t] : 0;
+    const unsigned at = scan_1024(v, ws, &total);
+    if (t < ntiles) tops[t] = carry + at;
+    carry += total;
+    __syncthreads();                     // ws and total are written again
+  }
+}
+
+// Every rating into its chunk's list. cursor: the chunks' starts (within
+// their scan tile), moved to their ends.
+template <int TO>
+__global__ void __launch_bounds__(256)
+k_bucket(int nb, const BlockMeta *__restrict__ meta, int64_t nnz,
+         const uint2 *__restrict__ where, const float *__restrict__ x,
+         const float *__restrict__ sub, const unsigned *__restrict__ tops,
+         unsigned *cursor, uint32_t *__restrict__ list, int32_t *flag) {
+  __shared__ float2 sub_lim[kTableBlocks];
+  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+    const Dest d = dest_of<TO>(meta, sub, b);
+    sub_lim[b] = make_float2(d.sub, d.lim);
+  }
+  __syncthreads();
+  int32_t bad = 0;
+  const int lane = threadIdx.x & 31;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31);
+       t0 < nnz; t0 += kRatings * stride) {
+    uint2 wh[kRatings];
+    float xx[kRatings];
+#pragma unroll
+    for (int k = 0; k < kRatings; ++k) {
+      const int64_t e = t0 + k * stride + lane;
+      wh[k] = e < nnz ? where[e] : make_uint2(kNowhere, 0);
+      xx[k] = e < nnz ? x[e] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < kRatings; ++k) {
+      const bool on = wh[k].x != kNowhere;
+      const int32_t slot = (int32_t)wh[k].x;
+      const unsigned at = chunk_add(cursor, on, slot);
+      if (!on) continue;
+      const float2 sl = sub_lim[wh[k].y >> 16];
+      const float y = __fsub_rn(xx[k], sl.x);
+      const uint32_t entry =
+          (wh[k].y & 0xffffu) |
+          (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(y)) << 16;
+      const int64_t pos = (int64_t)tops[slot / kScanTile] + at;
+      if (pos < nnz) list[pos] = entry;
+      if (TO == kToPlanes) bad |= plane_flags(y, sl.x, sl.y, xx[k]);
+    }
+  }
+  if (TO == kToPlanes) {
+    const int32_t all = __reduce_or_sync(0xffffffffu, bad);
+    if (all && lane == 0) atomicOr(flag, all);
+  }
+}
+
+// out: every cell of the planes (PLANES = 2: the offsets, then the mask).
+// The chunk in shared memory is zero between chunks: the cells that were set
+// are set back. Three CTAs an SM, so that two work while one's store drains.
+constexpr int kFillThreads = kPlaneChunk / 64;
+constexpr int kHold = 4;
+template <int PLANES>
+__global__ void __launch_bounds__(kFillThreads)
+k_fill(const BlockMeta *__restrict__ meta, int32_t nb, int32_t nchunks,
+       const unsigned *__restrict__ tops, const unsigned *__restrict__ ends,
+       uint32_t mask,
+       const uint32_t *__restrict__ list, __nv_bfloat16 *__restrict__ out) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  unsigned short *y = reinterpret_cast<unsigned short *>(smem);
+  unsigned short *mk = y + kPlaneChunk;
+  __shared__ int32_t ck0[kTableBlocks];
+  for (int b = threadIdx.x; b < nb; b += blockDim.x) ck0[b] = meta[b].ck0;
+  for (int e = threadIdx.x; e < PLANES * kPlaneChunk / 8; e += blockDim.x)
+    reinterpret_cast<uint4 *>(smem)[e] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+  auto edge = [&](int32_t slot) -> int64_t {    // where the list there ends
+    return (int64_t)tops[slot / kScanTile] + ends[slot];
+  };
+  struct Job {
+    int64_t from, to;
+    uint32_t v[kHold];                 // the first entries of this thread
+    __nv_bfloat16 *dst;                // thread 0: where the chunk goes
+    int64_t plane;
+    uint32_t bytes;
+  };
+  auto fetch = [&](int32_t ck) {
+    Job j;
+    j.from = j.to = 0;
+    if (ck >= nchunks) return j;
+    const int32_t slot = chunk_slot(ck, mask);
+    j.from = slot % kScanTile ? edge(slot - 1) : tops[slot / kScanTile];
+    j.to = edge(slot);
+    if (threadIdx.x == 0) {
+      const BlockMeta &bm = meta[upper_index(ck0, nb, ck)];
+      const int64_t c0 = (int64_t)(ck - bm.ck0) << kPlaneChunkLog;
+      j.plane = (int64_t)bm.s128 * bm.L_pad;
+      j.dst = out + bm.vx_off + c0;
+      // a plane is a multiple of 128 x 32 cells: whole 16-byte units
+      j.bytes = 2 * (uint32_t)min(j.plane - c0, (int64_t)kPlaneChunk);
+    }
+#pragma unroll
+    for (int h = 0; h < kHold; ++h) {
+      const int64_t e = j.from + h * kFillThreads + threadIdx.x;
+      if (e < j.to) j.v[h] = list[e];
+    }
+    return j;
+  };
+  auto put = [&](const Job &j, bool set) {
+    auto one = [&](uint32_t v) {
+      y[v & 0xffff] = set ? (unsigned short)(v >> 16) : 0;
+      if (PLANES == 2) mk[v & 0xffff] = set ? 0x3f80 : 0;        // 1
+    };
+#pragma unroll
+    for (int h = 0; h < kHold; ++h)
+      if (j.from + h * kFillThreads + threadIdx.x < j.to) one(j.v[h]);
+    for (int64_t e = j.from + kHold * kFillThreads + threadIdx.x; e < j.to;
+         e += kFillThreads)
+      one(list[e]);
+  };
+  Job job = fetch(blockIdx.x);
+  for (int32_t ck = blockIdx.x; ck < nchunks; ck += gridDim.x) {
+    put(job, true);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int p = 0; p < PLANES; ++p)
+        asm volatile(
+            "cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                job.dst + p * job.plane),
+            "r"((uint32_t)__cvta_generic_to_shared(y + p * kPlaneChunk)),
+            "r"(job.bytes)
+            : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
+    const Job next = fetch(ck + gridDim.x);
+    if (threadIdx.x == 0)
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    __syncthreads();
+    put(job, false);
+    job = next;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0)
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 int grid_for(int64_t n, int per_thread) {
@@ -375,17 +680,25 @@ cudaError_t launch_count(const GridDesc &g, int64_t nnz, const int32_t *u,
                          const int32_t *i, const float *x, int32_t nblocks,
                          unsigned long long *counts, long long *sums,
                          unsigned int *maxabs_bits, int32_t *err,
-                         cudaStream_t st) {
+                         cudaStream_t st, const BlockMeta *meta,
+                         unsigned *chunks, int64_t nchunks, uint2 *where) {
   if (nnz <= 0) return cudaSuccess;
+  const uint32_t mask = (uint32_t)(chunk_slots(nchunks) - 1);
   // big grids flush many per-CTA histograms: use fewer, longer CTAs
   int grid = grid_for(nnz, nblocks > 256 ? 16 : 4);
   const size_t sm = nblocks <= kSmemBlocks ? sizeof(CountTable) : 0;
-  if (fits_table(g))
-    k_count<true><<<grid, 256, sm, st>>>(g, nnz, u, i, x, nblocks, counts,
-                                         sums, maxabs_bits, err);
+  if (chunks)
+    k_count<true, true><<<grid, 256, sm + sizeof(Place) * kTableBlocks, st>>>(
+        g, nnz, u, i, x, nblocks, counts, sums, maxabs_bits, err, meta, chunks,
+        mask, where);
+  else if (fits_table(g))
+    k_count<true, false><<<grid, 256, sm, st>>>(
+        g, nnz, u, i, x, nblocks, counts, sums, maxabs_bits, err, meta, chunks,
+        mask, where);
   else
-    k_count<false><<<grid, 256, sm, st>>>(g, nnz, u, i, x, nblocks, counts,
-                                          sums, maxabs_bits, err);
+    k_count<false, false><<<grid, 256, sm, st>>>(
+        g, nnz, u, i, x, nblocks, counts, sums, maxabs_bits, err, meta, chunks,
+        mask, where);
   return cudaGetLastError();
 }
 
@@ -442,6 +755,69 @@ cudaError_t launch_scatter_planes(const GridDesc &g, const BlockMeta *meta,
                                   const float *shift, __nv_bfloat16 *VX,
                                   int32_t *flag, cudaStream_t st) {
   return scatter_to<kToPlanes>(g, meta, nnz, u, i, x, shift, VX, flag, st);
+}
+
+bool chunked_planes(const GridDesc &g, int64_t nnz, int64_t nchunks,
+                    int64_t plane_bytes, int64_t list_cap) {
+  return fits_table(g) && nnz > 0 && nnz <= list_cap && nnz < INT32_MAX &&
+         nchunks > 0 && nchunks <= (1 << 30) && plane_bytes >= kChunkedBytes;
+}
+
+int64_t chunk_slots(int64_t nchunks) {
+  int64_t n = 1;
+  while (n < nchunks) n *= 2;
+  return n;
+}
+
+int64_t chunk_words(int64_t nchunks) {
+  const int64_t n = chunk_slots(nchunks);
+  return n + (n + kScanTile - 1) / kScanTile;
+}
+
+template <int TO>
+static cudaError_t planes_to(const GridDesc &g, const BlockMeta *meta,
+                             int64_t nnz, const uint2 *where, const float *x,
+                             const float *sub, int32_t nchunks,
+                             unsigned *chunks, uint32_t *list,
+                             __nv_bfloat16 *out, int32_t *flag,
+                             cudaStream_t st) {
+  constexpr int PLANES = TO == kToPlanes ? 2 : 1;
+  constexpr int kBytes = PLANES * kPlaneChunk * 2;
+  const int32_t nslots = (int32_t)chunk_slots(nchunks);
+  const uint32_t mask = (uint32_t)nslots - 1;
+  const int ntiles = (nslots + kScanTile - 1) / kScanTile;
+  unsigned *tops = chunks + nslots;
+  k_chunk_scan<<<ntiles, 1024, 0, st>>>(nslots, chunks, tops);
+  k_chunk_tops<<<1, 1024, 0, st>>>(ntiles, tops);
+  k_bucket<TO><<<grid_for(nnz, 4), 256, 0, st>>>(
+      grid_blocks(g), meta, nnz, where, x, sub, tops, chunks, list, flag);
+  cudaError_t e = cudaFuncSetAttribute(
+      k_fill<PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+  if (e != cudaSuccess) return e;
+  const int per_sm = (215 << 10) / (kBytes + 2048 + 1024);
+  k_fill<PLANES><<<nchunks < 152 * per_sm ? nchunks : 152 * per_sm, kFillThreads,
+                   kBytes, st>>>(meta, grid_blocks(g), nchunks, tops, chunks,
+                                 mask, list, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_chunked_bf16(const GridDesc &g, const BlockMeta *meta,
+                                int64_t nnz, const uint2 *where, const float *x,
+                                const float *mu, int32_t nchunks,
+                                unsigned *chunks, uint32_t *list,
+                                __nv_bfloat16 *Wh, cudaStream_t st) {
+  return planes_to<kToBf16>(g, meta, nnz, where, x, mu, nchunks, chunks, list,
+                       Wh, nullptr, st);
+}
+
+cudaError_t launch_chunked_planes(const GridDesc &g, const BlockMeta *meta,
+                                  int64_t nnz, const uint2 *where, const float *x,
+                                  const float *shift, int32_t nchunks,
+                                  unsigned *chunks, uint32_t *list,
+                                  __nv_bfloat16 *VX, int32_t *flag,
+                                  cudaStream_t st) {
+  return planes_to<kToPlanes>(g, meta, nnz, where, x, shift, nchunks, chunks, list,
+                       VX, flag, st);
 }
 
 }  // namespace bsvd
