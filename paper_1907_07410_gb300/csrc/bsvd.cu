@@ -628,7 +628,8 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
                                   const int64_t *col_bounds,
                                   const int32_t *row_perm,
                                   const int32_t *col_perm, bool diag,
-                                  const Pieces *pieces = nullptr) {
+                                  const Pieces *pieces = nullptr,
+                                  bool own_perms = false) {
   if (!c) return BSVD_EINVAL;
   c->err.clear();
   c->sgd_ready = false;      // a new grid invalidates the SGD order
@@ -722,28 +723,35 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
                      cudaMemcpyHostToDevice, c->st), "partition");
 
   // permutations: copied into context memory, then checked on the device
+  // (own_perms: made here, from distinct sorted keys)
   c->has_rperm = row_perm != nullptr;
   c->has_cperm = col_perm != nullptr;
   CK(cudaMemsetAsync(c->d_err.p, 0, 2 * sizeof(int32_t), c->st), "partition");
   if (row_perm) {
     CK(c->d_rperm.ensure(sizeof(int32_t) * m), "partition");
-    CK(c->d_seen.ensure(sizeof(int32_t) * std::max(m, n)), "partition");
     CK(cudaMemcpyAsync(c->d_rperm.p, row_perm, sizeof(int32_t) * m,
                        cudaMemcpyDefault, c->st), "partition");
-    CK(launch_perm_check(c->d_rperm.as<int32_t>(), m, c->d_seen.as<int32_t>(),
-                         c->d_err.as<int32_t>(), c->st), "partition");
-    c->launches += 2;
+    if (!own_perms) {
+      CK(c->d_seen.ensure(sizeof(int32_t) * std::max(m, n)), "partition");
+      CK(launch_perm_check(c->d_rperm.as<int32_t>(), m,
+                           c->d_seen.as<int32_t>(), c->d_err.as<int32_t>(),
+                           c->st), "partition");
+      c->launches += 2;
+    }
   }
   if (col_perm) {
     CK(c->d_cperm.ensure(sizeof(int32_t) * n), "partition");
-    CK(c->d_seen.ensure(sizeof(int32_t) * std::max(m, n)), "partition");
     CK(cudaMemcpyAsync(c->d_cperm.p, col_perm, sizeof(int32_t) * n,
                        cudaMemcpyDefault, c->st), "partition");
-    CK(launch_perm_check(c->d_cperm.as<int32_t>(), n, c->d_seen.as<int32_t>(),
-                         c->d_err.as<int32_t>(), c->st), "partition");
-    c->launches += 2;
+    if (!own_perms) {
+      CK(c->d_seen.ensure(sizeof(int32_t) * std::max(m, n)), "partition");
+      CK(launch_perm_check(c->d_cperm.as<int32_t>(), n,
+                           c->d_seen.as<int32_t>(), c->d_err.as<int32_t>(),
+                           c->st), "partition");
+      c->launches += 2;
+    }
   }
-  if (row_perm || col_perm) {
+  if ((row_perm || col_perm) && !own_perms) {
     bsvd_status s = read_errors(c, "partition");
     if (s != BSVD_OK) return s;
   }
@@ -1135,7 +1143,7 @@ bsvd_status bsvd_partition_quantile(bsvd_ctx *c, int64_t m, int64_t n,
   return partition_impl(c, m, n, nnz, (const int32_t *)du, (const int32_t *)di,
                         (const float *)dx, p, q, rb.data(), cb.data(),
                         c->d_qperm.as<int32_t>(), c->d_qperm2.as<int32_t>(),
-                        false);
+                        false, nullptr, true);
 }
 
 static bsvd_status factor_impl(bsvd_ctx *c, int32_t k, const int32_t *ks);

@@ -60,8 +60,8 @@ cudaError_t launch_chunked_planes(const GridDesc &g, const BlockMeta *meta,
                                   int32_t *flag, cudaStream_t st);
 
 // ---- activity-quantile cut of one side (kernels_grid.cu) ----------------
-// Keys are padded to quantile_cut_padded(size) entries. counts: size,
-// keys: padded, cum: size + 1, perm: size, bounds: parts + 1 (device).
+// counts: size, keys: quantile_cut_padded(size) (the sort's work included),
+// cum: size + 1, perm: size, bounds: parts + 1 (device).
 // *launches is increased by the number of kernels queued.
 int64_t quantile_cut_padded(int64_t size);
 cudaError_t launch_quantile_cut(const int32_t *ids, int64_t nnz, int64_t size,
