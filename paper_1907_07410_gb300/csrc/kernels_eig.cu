@@ -506,10 +506,13 @@ __device__ int onesided_jacobi(float (*Ac)[P], float (*Vc)[P], int n,
           float na[RPL], nb[RPL], nva[RPL], nvb[RPL];
 #pragma unroll
           for (int h = 0; h < RPL; ++h) {
-            na[h] = c * a[h] - s * b[h];
-            nb[h] = s * a[h] + c * b[h];
-            nva[h] = c * va[h] - s * vb[h];
-            nvb[h] = s * va[h] + c * vb[h];
+            // which product is rounded first is written out, so that a change
+            // of the code around it changes no result
+            na[h] = fmaf(c, a[h], -__fmul_rn(s, b[h]));
+            nb[h] = B == 16 ? fmaf(c, b[h], __fmul_rn(s, a[h]))
+                            : fmaf(s, a[h], __fmul_rn(c, b[h]));
+            nva[h] = fmaf(c, va[h], -__fmul_rn(s, vb[h]));
+            nvb[h] = fmaf(s, va[h], __fmul_rn(c, vb[h]));
           }
           st_vec(ap, na);
           st_vec(aq, nb);
