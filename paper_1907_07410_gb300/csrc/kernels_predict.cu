@@ -17,6 +17,7 @@ namespace bsvd {
 namespace {
 
 constexpr int kPredictThreads = 256;
+constexpr int64_t kFewQueries = 40000;   // about eight lanes each in one wave
 constexpr int kSqerrThreads = 512;   // 304 CTAs of them fill the SMs
 
 // Where a query's block keeps what a prediction reads. A CTA copies the
@@ -176,6 +177,51 @@ k_predict(PredictArgs a, int64_t nq, const int32_t *__restrict__ u,
   if (bad) atomicOr(err, bad);
 }
 
+// Few queries: LPQ lanes take one query from its ids to its sum, so every load
+// of the call is under way at once and no CTA fills a table first. The chunks
+// of a row and the tree of its sum are those of predict_warp: the same bits.
+// A call of 2,000 / 20,000 queries, kp = 40 on an 8 x 4 quantile grid: 24 / 26
+// us, 31 / 31 by k_predict; kp = 56, 13 x 9 equal blocks 22 / 24, 31 / 31. From
+// 40,000 on both take the same, and from 400,000 on the table wins.
+template <int LPQ>
+__global__ void __launch_bounds__(kPredictThreads)
+k_predict_few(PredictArgs a, int64_t nq, const int32_t *__restrict__ u,
+              const int32_t *__restrict__ it, float *__restrict__ yhat,
+              int32_t *err) {
+  const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LPQ;
+  const int sub = threadIdx.x % LPQ, n4 = a.kp / 4;
+  const bool in = t < nq;
+  int32_t blk = 0, r = 0, c = 0;
+  const bool ok = in && locate(a.g, u[t], it[t], &blk, &r, &c);
+  float mu = 0.f, dot = 0.f;
+  if (ok) {
+    const BlockMeta &bm = a.meta[blk];
+    mu = a.mu[blk];
+    if (bm.keff > 0 && (bm.owned || !a.owned_only)) {
+      const float4 *fs = reinterpret_cast<const float4 *>(
+          a.Fs + bm.fs_off + (int64_t)(bm.trans ? c : r) * a.kp);
+      const float4 *fl = reinterpret_cast<const float4 *>(
+          a.FL + bm.fl_off + (int64_t)(bm.trans ? r : c) * a.kp);
+#pragma unroll 4
+      for (int j = sub; j < n4; j += LPQ) {
+        const float4 p = __ldg(fs + j), v = __ldg(fl + j);
+        dot = fmaf(p.x, v.x, dot);
+        dot = fmaf(p.y, v.y, dot);
+        dot = fmaf(p.z, v.z, dot);
+        dot = fmaf(p.w, v.w, dot);
+      }
+    }
+  }
+#pragma unroll
+  for (int o = LPQ / 2; o > 0; o >>= 1)
+    dot += __shfl_xor_sync(0xffffffffu, dot, o);
+  if (!in || sub != 0) return;
+  float y = mu + dot;
+  if (a.clamp) y = fminf(fmaxf(y, a.lo), a.hi);
+  yhat[t] = ok ? y : 0.f;
+  if (!ok) atomicOr(err, kErrIndex);
+}
+
 // With a.owned_only, queries in blocks this context does not hold are
 // skipped; the CTA's count of summed queries goes to counts.
 template <int LPQ, bool TABLE>
@@ -284,6 +330,12 @@ cudaError_t launch_predict(const PredictArgs &a, int64_t nq, const int32_t *u,
   return by_shape(a, [&](auto l, auto tb) {
     constexpr int LPQ = decltype(l)::value;
     constexpr bool TB = decltype(tb)::value;
+    if (nq <= kFewQueries) {
+      const int64_t ctas = (nq * LPQ + kPredictThreads - 1) / kPredictThreads;
+      k_predict_few<LPQ><<<(unsigned)ctas, kPredictThreads, 0, st>>>(
+          a, nq, u, i, yhat, err);
+      return cudaGetLastError();
+    }
     k_predict<LPQ, TB><<<grid_for(nq), kPredictThreads, TB ? sizeof(Table) : 0,
                          st>>>(a, nq, u, i, yhat, err);
     return cudaGetLastError();

@@ -151,3 +151,34 @@ def test_squared_errors_skip_blocks_of_another_shard():
     assert np.array_equal(y[~mine].astype(np.float32), mu[blk[~mine]])
     want = np.sum((y[mine] - r.x_test[mine]) ** 2)
     assert abs(s - want) <= 1e-12 * want
+
+
+@pytest.mark.parametrize("k", [3, 10, 20, 40, 56])
+@pytest.mark.parametrize("grid", ["equal", "quantile", "diag"])
+def test_few_queries_equal_many(k, grid):
+    """A short call takes the form with several lanes per query from the ids
+    on; its sums are those of the long call, bit for bit."""
+    rng = np.random.default_rng(k)
+    m, n, nnz = 700, 300, 9000
+    cells = rng.permutation(m * n)[:nnz]
+    u, i = (cells // n).astype(np.int32), (cells % n).astype(np.int32)
+    x = rng.integers(1, 6, nnz).astype(np.float32)
+    with bs.Context() as ctx:
+        if grid == "quantile":
+            ctx.partition_quantile(m, n, u, i, x, 3, 2)
+        elif grid == "equal":
+            ctx.partition(m, n, u, i, x, 3, 2)
+        else:
+            keep = (u < 400) == (i < 100)
+            ctx.partition_diag([0, 400, 700], [0, 100, 300], u[keep], i[keep],
+                               x[keep])
+        ctx.factor(k, warn=False)
+        q = rng.integers(0, m * n, 40001 + 37)
+        qu, qi = (q // n).astype(np.int32), (q % n).astype(np.int32)
+        if grid == "diag":
+            qi = np.where(qu < 400, qi % 100, 100 + qi % 200).astype(np.int32)
+        many = ctx.predict(qu, qi)
+        for nq in (1, 3, 4, 5, 31, 33, 1000, 40000):
+            assert np.array_equal(ctx.predict(qu[:nq], qi[:nq]), many[:nq]), nq
+        with pytest.raises(bs.BsvdError):
+            ctx.predict(np.array([0, m], np.int32), np.array([0, 0], np.int32))
