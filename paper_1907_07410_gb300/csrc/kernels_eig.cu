@@ -319,12 +319,32 @@ __device__ __forceinline__ void st_vec(float *p, const float (&v)[N]) {
 // Partial S = X^T X and H = X^T Z over one chunk of up to kChunkRows rows,
 // for every chunk of every running block; k_rr_solve sums a block's chunks
 // in a fixed order, so the totals do not depend on scheduling. The 256
-// threads form a 16 x 16 grid over the b x b outputs, each thread a TI x TI
-// register tile (TI = b / 16): per row, three 16-byte shared loads (its
-// slices of the X row for i and j, and of the Z row for j) feed 2 TI^2
+// threads form a 16 x 16 grid over the b x b outputs, each thread a TI x TJ
+// register tile (TJ = b / 16): per row, three 16-byte shared loads (its
+// slices of the X row for i and j, and of the Z row for j) feed 2 TI TJ
 // fused multiply-adds. The rows are added in order, 32 at a time staged in
 // shared memory.
-template <int B>
+// SPLIT: few chunks leave the chip idle, so 2 SPLIT CTAs take a chunk, each
+// B / SPLIT rows of S or of H (each output the same sum in the same order).
+// The rows come through a ring of passes (cp.async): loaded at the
+// start of its own pass, every pass waited for the L2. 16 blocks of 1,000 rows
+// at b = 32: 27 us before both, 14 now; 16 of 1,500 rows at b = 64: 55, 37; 256
+// blocks of 250 rows, whole chunks: 15 (cold caches).
+constexpr int kSgRows = 32;                  // rows per pass
+// more passes under way where a CTA has an SM for itself
+template <int SPLIT>
+constexpr int kSgStagesOf = SPLIT ? 4 : 3;
+template <int B, int SPLIT>
+constexpr size_t small_gram_smem() {
+  return sizeof(float) * 2 * kSgRows * B * kSgStagesOf<SPLIT>;
+}
+__device__ __forceinline__ void cp_async16(float *dst, const float *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+template <int B, int SPLIT>
 __global__ void __launch_bounds__(256)
 k_small_gram(const BlockMeta *__restrict__ meta,
              const SolverState *__restrict__ state,
@@ -332,56 +352,83 @@ k_small_gram(const BlockMeta *__restrict__ meta,
              const float *__restrict__ Z, float *__restrict__ SHp) {
   pdl_wait();
   pdl_trigger();
-  constexpr int TI = B / 16;
-  constexpr int SR = 32;                   // rows staged per pass
-  __shared__ __align__(16) float Xs[SR][B];
-  __shared__ __align__(16) float Zs[SR][B];
+  constexpr int TJ = B / 16, TI = SPLIT ? TJ / SPLIT : TJ;
+  constexpr int SR = kSgRows;
+  constexpr int kSgStages = kSgStagesOf<SPLIT>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float (*ring)[2][SR][B] = reinterpret_cast<float (*)[2][SR][B]>(smem_raw);
   const int2 t = chunks[blockIdx.x];
   if (state[t.x].status != kRunning) return;
+  const bool do_s = !SPLIT || blockIdx.y < SPLIT;
+  const bool do_h = !SPLIT || blockIdx.y >= SPLIT;
   const BlockMeta bm = meta[t.x];
   const int rows = min(kChunkRows, bm.s - t.y);
   const float *Xb = X + bm.x_off + (int64_t)t.y * B;
   const float *Zb = Z + bm.x_off + (int64_t)t.y * B;
-  const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
-  float sa[TI][TI], ha[TI][TI];
+  const int tj = threadIdx.x & 15;
+  const int i0 = (SPLIT ? (int)blockIdx.y % SPLIT * (B / SPLIT) : 0) +
+                 TI * ((int)threadIdx.x >> 4);
+  float sa[TI][TJ], ha[TI][TJ];
 #pragma unroll
   for (int a = 0; a < TI; ++a)
 #pragma unroll
-    for (int b = 0; b < TI; ++b) sa[a][b] = ha[a][b] = 0.f;
-  for (int r0 = 0; r0 < rows; r0 += SR) {
-    const int nr = min(SR, rows - r0);
-    __syncthreads();                       // the last pass has read Xs, Zs
-    for (int e4 = threadIdx.x; e4 < nr * (B / 4); e4 += 256) {
-      const int64_t o = (int64_t)r0 * B + 4 * e4;
-      reinterpret_cast<float4 *>(&Xs[0][0])[e4] =
-          *reinterpret_cast<const float4 *>(Xb + o);
-      reinterpret_cast<float4 *>(&Zs[0][0])[e4] =
-          *reinterpret_cast<const float4 *>(Zb + o);
+    for (int b = 0; b < TJ; ++b) sa[a][b] = ha[a][b] = 0.f;
+  const int passes = (rows + SR - 1) / SR;
+  auto load = [&](int p) {                   // a group of copies, maybe empty
+    if (p < passes) {
+      const int n4 = min(SR, rows - p * SR) * (B / 4);
+      const float *xs = Xb + (int64_t)p * SR * B, *zs = Zb + (int64_t)p * SR * B;
+      for (int e = threadIdx.x; e < n4; e += 256) {
+        cp_async16(&ring[p % kSgStages][0][0][0] + 4 * e, xs + 4 * e);
+        if (do_h) cp_async16(&ring[p % kSgStages][1][0][0] + 4 * e, zs + 4 * e);
+      }
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int p = 0; p < kSgStages - 1; ++p) load(p);
+  for (int p = 0; p < passes; ++p) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kSgStages - 2) : "memory");
+    // pass p is there for all, and pass p - 1 read by all
     __syncthreads();
-    for (int rr = 0; rr < nr; ++rr) {
-      float xi[TI], xj[TI], zj[TI];
-      ld_vec(&Xs[rr][TI * ti], xi);
-      ld_vec(&Xs[rr][TI * tj], xj);
-      ld_vec(&Zs[rr][TI * tj], zj);
+    load(p + kSgStages - 1);
+    const float (*Xs)[B] = ring[p % kSgStages][0];
+    const float (*Zs)[B] = ring[p % kSgStages][1];
+    const int nr = min(SR, rows - p * SR);
+    // which sums: known to the compiler, so that the rows' loads run ahead
+    auto sums = [&](auto s, auto h) {
+      auto add = [&](int rr) {
+        float xi[TI], xj[TJ], zj[TJ];
+        ld_vec(&Xs[rr][i0], xi);
+        if (s.value) ld_vec(&Xs[rr][TJ * tj], xj);
+        if (h.value) ld_vec(&Zs[rr][TJ * tj], zj);
 #pragma unroll
-      for (int a = 0; a < TI; ++a)
+        for (int a = 0; a < TI; ++a)
 #pragma unroll
-        for (int b = 0; b < TI; ++b) {
-          sa[a][b] = fmaf(xi[a], xj[b], sa[a][b]);
-          ha[a][b] = fmaf(xi[a], zj[b], ha[a][b]);
-        }
-    }
+          for (int b = 0; b < TJ; ++b) {
+            if (s.value) sa[a][b] = fmaf(xi[a], xj[b], sa[a][b]);
+            if (h.value) ha[a][b] = fmaf(xi[a], zj[b], ha[a][b]);
+          }
+      };
+      if (nr == SR) {
+#pragma unroll 8
+        for (int rr = 0; rr < SR; ++rr) add(rr);
+      } else {
+        for (int rr = 0; rr < nr; ++rr) add(rr);
+      }
+    };
+    if (!SPLIT) sums(std::true_type(), std::true_type());
+    else if (do_s) sums(std::true_type(), std::false_type());
+    else sums(std::false_type(), std::true_type());
   }
   float *S = SHp + (int64_t)blockIdx.x * 2 * B * B;
   float *H = S + B * B;
 #pragma unroll
   for (int a = 0; a < TI; ++a)
 #pragma unroll
-    for (int b = 0; b < TI; ++b) {
-      const int idx = (TI * ti + a) * B + TI * tj + b;
-      S[idx] = sa[a][b];
-      H[idx] = ha[a][b];
+    for (int b = 0; b < TJ; ++b) {
+      const int idx = (i0 + a) * B + TJ * tj + b;
+      if (do_s) S[idx] = sa[a][b];
+      if (do_h) H[idx] = ha[a][b];
     }
 }
 
@@ -1276,8 +1323,16 @@ cudaError_t launch_small_gram(const EigBuffers &e, const int2 *chunks,
   if (nchunks <= 0) return cudaSuccess;
   return by_width(e.bsub, [&](auto w) {
     constexpr int B = decltype(w)::value;
-    return launch_pdl(k_small_gram<B>, dim3(nchunks), dim3(256), 0, st, e.meta,
-                      e.state, chunks, (const float *)e.X,
+    // a wave of split CTAs, or whole chunks
+    constexpr int SPLIT = B / 16;
+    const bool split = (int64_t)nchunks * 2 * SPLIT <= 4 * (int64_t)e.nsm;
+    auto kernel = split ? k_small_gram<B, SPLIT> : k_small_gram<B, 0>;
+    const size_t sm = split ? small_gram_smem<B, SPLIT>() : small_gram_smem<B, 0>();
+    const cudaError_t err = cudaFuncSetAttribute(
+        kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (err != cudaSuccess) return err;
+    return launch_pdl(kernel, dim3(nchunks, split ? 2 * SPLIT : 1), dim3(256),
+                      sm, st, e.meta, e.state, chunks, (const float *)e.X,
                       (const float *)e.Z, e.SH);
   });
 }
