@@ -796,12 +796,10 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
     CK(device_view(c, x, sizeof(float) * nnz, c->s_c, &dx), "partition");
   }
 
-  CK(cudaMemsetAsync(c->d_counts.p, 0, sizeof(unsigned long long) * nb, c->st),
-     "partition");
-  CK(cudaMemsetAsync(c->d_sums.p, 0, sizeof(long long) * nb, c->st),
-     "partition");
-  CK(cudaMemsetAsync(c->d_maxabs.p, 0, sizeof(unsigned int), c->st),
-     "partition");
+  CK(launch_clear(nb, c->d_counts.as<unsigned long long>(),
+                  c->d_sums.as<long long>(), c->d_maxabs.as<unsigned int>(),
+                  c->st), "partition");
+  ++c->launches;
   const GridDesc g = c->grid();
   // Large planes are filled chunk by chunk; the lists on the way take the
   // place of the float32 arena, which such a partition does not hold (or
@@ -841,10 +839,16 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
                   c->d_sums.as<long long>(), c->d_maxabs.as<unsigned int>(),
                   c->d_err.as<int32_t>(), c->st, c->d_meta.as<BlockMeta>(),
                   chunks, nchunks, where), "partition: count");
+  if (c->tc_planes) {
+    CK(c->d_shift.ensure(sizeof(float) * nb), "partition");
+    CK(c->d_delta.ensure(sizeof(float) * nb), "partition");
+  }
   CK(launch_means(nb, c->d_counts.as<unsigned long long>(),
                   c->d_sums.as<long long>(), c->d_maxabs.as<unsigned int>(),
-                  c->d_mu.as<float>(), c->d_err.as<int32_t>(), c->st),
-     "partition: means");
+                  c->d_mu.as<float>(),
+                  c->tc_planes ? c->d_shift.as<float>() : nullptr,
+                  c->tc_planes ? c->d_delta.as<float>() : nullptr,
+                  c->d_err.as<int32_t>(), c->st), "partition: means");
   c->launches += nnz > 0 ? 2 : 1;
   if (c->w32) {
     const bsvd_status ws = write_w();
@@ -870,11 +874,6 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
   // bf16 planes for the exact tensor-core Gram
   c->tc_exact = false;
   if (c->tc_planes) {
-    CK(c->d_shift.ensure(sizeof(float) * nb), "partition");
-    CK(c->d_delta.ensure(sizeof(float) * nb), "partition");
-    CK(launch_plane_shift(nb, c->d_counts.as<unsigned long long>(),
-                          c->d_sums.as<long long>(), c->d_shift.as<float>(),
-                          c->d_delta.as<float>(), c->st), "partition: shift");
     int32_t *found = c->d_err.as<int32_t>() + 1;
     CK(chunked
            ? launch_chunked_planes(g, c->d_meta.as<BlockMeta>(), nnz, where,
@@ -886,7 +885,7 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
                                    (const float *)dx, c->d_shift.as<float>(),
                                    c->d_VX.as<__nv_bfloat16>(), found, c->st),
        "partition: planes");
-    c->launches += chunked ? 5 : nnz > 0 ? 2 : 1;
+    c->launches += chunked ? 4 : nnz > 0;
   }
   mark(c, 1);
   int32_t flag = 0;

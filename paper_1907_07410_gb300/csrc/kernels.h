@@ -22,10 +22,16 @@ cudaError_t launch_count(const GridDesc &g, int64_t nnz, const int32_t *u,
                          cudaStream_t st, const BlockMeta *meta = nullptr,
                          unsigned *chunks = nullptr, int64_t nchunks = 0,
                          uint2 *where = nullptr);
+// Zero what launch_count adds to.
+cudaError_t launch_clear(int32_t nblocks, unsigned long long *counts,
+                         long long *sums, unsigned int *maxabs_bits,
+                         cudaStream_t st);
+// shift, delta (both or none): the planes' round(mu) and mu - round(mu)
 cudaError_t launch_means(int32_t nblocks, const unsigned long long *counts,
                          const long long *sums,
                          const unsigned int *maxabs_bits, float *mu,
-                         int32_t *err, cudaStream_t st);
+                         float *shift, float *delta, int32_t *err,
+                         cudaStream_t st);
 // Centred cells into the zeroed float32 arena, or their bf16 rounding into the
 // zeroed bf16 blocks.
 cudaError_t launch_scatter(const GridDesc &g, const BlockMeta *meta,
@@ -98,10 +104,6 @@ cudaError_t launch_gram_bf16(const BlockMeta *meta, const int4 *tiles,
                              int32_t *err, cudaStream_t st);
 
 // ---- bf16 planes for the tensor-core Gram (kernels_partition.cu) ----------
-// shift[b] = round(mu_b) (exact mean from the sums), delta[b] = mu_b - shift.
-cudaError_t launch_plane_shift(int32_t nblocks, const unsigned long long *counts,
-                               const long long *sums, float *shift,
-                               float *delta, cudaStream_t st);
 // Y = x - shift, M = 1 at every rating, into the zeroed planes. *flag gets
 // kErrNotExact when some x - shift is not an integer small enough
 // (|y|^2 L_pad < 2^24, |y| <= 256) for the tensor-core Gram to be exact,

@@ -267,58 +267,69 @@ k_count(GridDesc g, int64_t nnz, const int32_t *__restrict__ u,
   if (threadIdx.x == 0 && s_max) atomicMax(maxabs_bits, s_max);
 }
 
+__global__ void __launch_bounds__(256)
+k_clear(int32_t nblocks, unsigned long long *counts, long long *sums,
+        unsigned int *maxabs_bits) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b < nblocks) {
+    counts[b] = 0;
+    sums[b] = 0;
+  }
+  if (b == 0) *maxabs_bits = 0;
+}
+
+// The block means, and for the planes (shift != null) the rounded mean and
+// what it leaves. One CTA of as many warps as the blocks need; the totals by
+// shuffles (ten barriers of 1,024 threads took longer than the rest: 7.5 us,
+// now 3.3, the rounded means included).
 __global__ void __launch_bounds__(1024)
 k_means(int32_t nblocks, const unsigned long long *counts,
         const long long *sums, const unsigned int *maxabs_bits, float *mu,
-        int32_t *err) {
-  __shared__ unsigned long long s_c[1024];
-  __shared__ long long s_s[1024];
+        float *shift, float *delta, int32_t *err) {
+  __shared__ unsigned long long s_c[32];
+  __shared__ long long s_s[32];
   unsigned long long c = 0;
   long long s = 0;
   for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
     c += counts[b];
     s += sums[b];
   }
-  s_c[threadIdx.x] = c;
-  s_s[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      s_c[threadIdx.x] += s_c[threadIdx.x + w];
-      s_s[threadIdx.x] += s_s[threadIdx.x + w];
-    }
-    __syncthreads();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    c += __shfl_xor_sync(0xffffffffu, c, o);
+    s += __shfl_xor_sync(0xffffffffu, s, o);
   }
-  const unsigned long long total_c = s_c[0];
-  const long long total_s = s_s[0];
+  if ((threadIdx.x & 31) == 0) {
+    s_c[threadIdx.x >> 5] = c;
+    s_s[threadIdx.x >> 5] = s;
+  }
+  __syncthreads();
+  unsigned long long total_c = 0;
+  long long total_s = 0;
+  for (int w = 0; w < (int)blockDim.x / 32; ++w) {
+    total_c += s_c[w];
+    total_s += s_s[w];
+  }
   const double xmax = (double)__uint_as_float(*maxabs_bits);
   // |sum| <= count * max|x| * 2^32 must stay inside int64
   if ((double)total_c * xmax >= 2147483648.0) {
     if (threadIdx.x == 0) atomicOr(err, kErrSumRange);
   }
-  float gmean = 0.0f;
-  if (total_c)
-    gmean = __double2float_rn(__ddiv_rn(__dmul_rn((double)total_s, 0x1p-32),
-                                        (double)total_c));
   for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-    unsigned long long cb = counts[b];
-    mu[b] = cb ? __double2float_rn(__ddiv_rn(
-                     __dmul_rn((double)sums[b], 0x1p-32), (double)cb))
-               : gmean;
-  }
-}
-
-__global__ void __launch_bounds__(256)
-k_plane_shift(int32_t nblocks, const unsigned long long *counts,
-              const long long *sums, float *shift, float *delta) {
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nblocks;
-       b += gridDim.x * blockDim.x) {
     const unsigned long long cb = counts[b];
-    double mu = 0.0;
-    if (cb) mu = __ddiv_rn(__dmul_rn((double)sums[b], 0x1p-32), (double)cb);
-    const double c = rint(mu);
-    shift[b] = (float)c;
-    delta[b] = __double2float_rn(mu - c);
+    // an empty block's mean is the mean of all ratings (0 without any)
+    const unsigned long long over = cb ? cb : total_c;
+    double m = 0.0;
+    if (over)
+      m = __ddiv_rn(__dmul_rn((double)(cb ? sums[b] : total_s), 0x1p-32),
+                    (double)over);
+    mu[b] = __double2float_rn(m);
+    if (shift) {
+      if (!cb) m = 0.0;
+      const double r = rint(m);
+      shift[b] = (float)r;
+      delta[b] = __double2float_rn(m - r);
+    }
   }
 }
 
@@ -658,15 +669,6 @@ int grid_for(int64_t n, int per_thread) {
 
 }  // namespace
 
-cudaError_t launch_plane_shift(int32_t nblocks, const unsigned long long *counts,
-                               const long long *sums, float *shift,
-                               float *delta, cudaStream_t st) {
-  if (nblocks <= 0) return cudaSuccess;
-  k_plane_shift<<<(nblocks + 255) / 256, 256, 0, st>>>(nblocks, counts, sums,
-                                                       shift, delta);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_perm_check(const int32_t *perm, int64_t n, int32_t *seen,
                               int32_t *err, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(seen, 0, sizeof(int32_t) * n, st);
@@ -710,11 +712,23 @@ cudaError_t launch_stack_ids(int64_t nnz, int32_t nb, const int64_t *starts,
   return cudaGetLastError();
 }
 
+cudaError_t launch_clear(int32_t nblocks, unsigned long long *counts,
+                         long long *sums, unsigned int *maxabs_bits,
+                         cudaStream_t st) {
+  k_clear<<<nblocks / 256 + 1, 256, 0, st>>>(nblocks, counts, sums,
+                                             maxabs_bits);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_means(int32_t nblocks, const unsigned long long *counts,
                          const long long *sums,
                          const unsigned int *maxabs_bits, float *mu,
-                         int32_t *err, cudaStream_t st) {
-  k_means<<<1, 1024, 0, st>>>(nblocks, counts, sums, maxabs_bits, mu, err);
+                         float *shift, float *delta, int32_t *err,
+                         cudaStream_t st) {
+  int threads = (nblocks + 31) / 32 * 32;
+  threads = threads < 32 ? 32 : threads > 1024 ? 1024 : threads;
+  k_means<<<1, threads, 0, st>>>(nblocks, counts, sums, maxabs_bits, mu, shift,
+                                 delta, err);
   return cudaGetLastError();
 }
 
