@@ -5,18 +5,18 @@
 // fixed point with 32 fraction bits (x * 2^32), so the totals are exact
 // integers and do not depend on the order of the atomic adds.
 // Pass 2 (k_means) turns the totals into mu_b = fl32(fl64(sum) / count).
-// Pass 3 (k_scatter, or k_scatter_planes for the exact tensor-core Gram)
-// writes fl32(x - mu_b), or its bf16 rounding, or the bf16 offset and the
-// observation mask, into the zeroed dense blocks.
+// Pass 3 writes fl32(x - mu_b), or its bf16 rounding, or the bf16 offset and
+// the observation mask: k_scatter into zeroed dense blocks, or for large
+// planes k_bucket and k_fill, which write every cell once.
 //
 // Every pass looks up a block per rating. A CTA keeps the grid's bounds and
 // what it needs of each block in shared memory (BoundsTable, Dest); from
 // global memory a rating's six or more lookups touch up to 32 lines per warp
 // each. A thread takes kRatings ratings at a time, so that their loads
-// overlap: counting 90 million ratings into 256 blocks takes 0.87 ms (1.43
-// before both). The scatter of that many into 17 GB of bf16 cells stays at 3.2
-// to 3.8 ms: each 2-byte write is a 32-byte sector of its own that DRAM reads
-// and writes, about 28 billion a second at any number of ratings in flight.
+// overlap: counting 90 million ratings into 256 blocks takes 0.90 ms (1.43
+// before both). A random access of the L2 a rating (the position of an id, a
+// counter, a list's place) takes about 75 us per ten million, which is what
+// the counting and listing of a large matrix are bound by.
 #include <type_traits>
 
 #include "kernels.h"
