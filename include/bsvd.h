@@ -381,8 +381,8 @@ bsvd_status bsvd_factor_report(bsvd_ctx *ctx, int32_t *iters,
  *   ms[2] subspace iteration (eigen-solve)    ms[3] projection and norms
  *   ms[4] prediction / squared-error sum
  *   ms[5] inside ms[2]: the tensor-core panel products' own device time
- *         (each launch's span, first CTA start to last CTA end, summed on
- *         the device; 0 on the FP32 SIMT panel path)
+ *         (each launch's span, first CTA start to last CTA end, taken on
+ *         the device, summed; 0 on the FP32 SIMT panel path)
  *   ms[6] inside ms[2]: Rayleigh-Ritz kernels (Grams, solve, rotate,
  *         check); with the loop in a graph, the rest of ms[2]
  *   ms[7] the rest of ms[2] (start basis, host round trips between steps)
