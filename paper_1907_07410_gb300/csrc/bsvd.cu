@@ -115,7 +115,7 @@ struct bsvd_ctx {
   int32_t *d_run_host = nullptr;  // the same memory seen from the device
   int32_t run_seq = 0;
   int32_t n_ptiles = 0;
-  std::vector<CUtensorMap> h_gmaps, h_xmaps, h_pwmaps;
+  std::vector<CUtensorMap> h_maps, h_gmaps, h_xmaps, h_pwmaps;
   // tensor-core projection: 128-column tiles of W and one TMA map per block
   DevBuf d_pjtiles, d_pwmaps;
   int32_t n_pjtiles = 0;
@@ -888,6 +888,33 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
     c->launches += chunked ? 4 : nnz > 0;
   }
   mark(c, 1);
+  // one TMA map per block over its bf16 rows, [Y; M] or the bf16 W, encoded
+  // and sent while the device fills the planes
+  EncodeTiledFn enc = planes ? tensor_map_encoder() : nullptr;
+  CUresult encoded = CUDA_SUCCESS;
+  if (enc) {
+    const int64_t plane_rows = c->cfg.precision == BSVD_BF16 ? 1 : 2;
+    c->h_maps.assign(nb, CUtensorMap());
+    for (int32_t b = 0; b < nb && encoded == CUDA_SUCCESS; ++b) {
+      const BlockMeta &bm = c->meta[b];
+      if (bm.s == 0 || !bm.owned) continue;
+      cuuint64_t dims[2] = {(cuuint64_t)bm.L_pad,
+                            (cuuint64_t)(plane_rows * bm.s128)};
+      cuuint64_t strides[1] = {(cuuint64_t)bm.L_pad * 2};
+      cuuint32_t box[2] = {64, 128};
+      cuuint32_t es[2] = {1, 1};
+      encoded = enc(&c->h_maps[b], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                    c->d_VX.as<__nv_bfloat16>() + bm.vx_off, dims, strides,
+                    box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_128B,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    }
+    CK(c->d_maps.ensure(sizeof(CUtensorMap) * nb), "partition");
+    // stream-ordered: the context's stream may be a non-blocking one
+    CK(cudaMemcpyAsync(c->d_maps.p, c->h_maps.data(), sizeof(CUtensorMap) * nb,
+                       cudaMemcpyHostToDevice, c->st), "partition");
+  }
   int32_t flag = 0;
   bsvd_status s = read_errors(c, "partition", &flag);
   if (s != BSVD_OK) return s;
@@ -905,37 +932,10 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
   }
   take(c, 0, 0, 1);
   if ((c->tc_planes && c->tc_exact) || c->cfg.precision == BSVD_BF16) {
-    const int64_t plane_rows = c->cfg.precision == BSVD_BF16 ? 1 : 2;
-    {
-      // one TMA map per block over its bf16 rows: [Y; M] or the bf16 W
-      EncodeTiledFn enc = tensor_map_encoder();
-      if (!enc) return fail(c, BSVD_ECUDA, "partition: no cuTensorMapEncodeTiled");
-      std::vector<CUtensorMap> maps(nb);
-      std::memset(maps.data(), 0, sizeof(CUtensorMap) * nb);
-      for (int32_t b = 0; b < nb; ++b) {
-        const BlockMeta &bm = c->meta[b];
-        if (bm.s == 0 || !bm.owned) continue;
-        cuuint64_t dims[2] = {(cuuint64_t)bm.L_pad,
-                              (cuuint64_t)(plane_rows * bm.s128)};
-        cuuint64_t strides[1] = {(cuuint64_t)bm.L_pad * 2};
-        cuuint32_t box[2] = {64, 128};
-        cuuint32_t es[2] = {1, 1};
-        CUresult r = enc(&maps[b], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
-                         c->d_VX.as<__nv_bfloat16>() + bm.vx_off, dims,
-                         strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                         CU_TENSOR_MAP_SWIZZLE_128B,
-                         CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS)
-          return fail(c, BSVD_ECUDA, "partition: tensor map %d failed (%d)", b,
-                      (int)r);
-      }
-      CK(c->d_maps.ensure(sizeof(CUtensorMap) * nb), "partition");
-      // stream-ordered: the context's stream may be a non-blocking one
-      CK(cudaMemcpyAsync(c->d_maps.p, maps.data(), sizeof(CUtensorMap) * nb,
-                         cudaMemcpyHostToDevice, c->st), "partition");
-      CK(cudaStreamSynchronize(c->st), "partition");
-    }
+    if (!enc) return fail(c, BSVD_ECUDA, "partition: no cuTensorMapEncodeTiled");
+    if (encoded != CUDA_SUCCESS)
+      return fail(c, BSVD_ECUDA, "partition: tensor maps failed (%d)",
+                  (int)encoded);
   }
   if (c->cfg.precision == BSVD_TF32) {
     // one TMA map per block over its float32 W (s_pad x L_pad)
@@ -1021,16 +1021,15 @@ bsvd_status bsvd_partition_batch(bsvd_ctx *c, int32_t nb,
 }
 
 // One side of the activity-quantile grid: perm (host or device, size
-// entries) and bounds (host, parts + 1).
+// entries), and bounds on the device (parts + 1).
 static bsvd_status quantile_side(bsvd_ctx *c, const char *what, int64_t size,
                                  int64_t nnz, const int32_t *ids,
                                  int32_t parts, int32_t *perm,
-                                 int64_t *bounds) {
+                                 int64_t *dbounds) {
   const int64_t padded = quantile_cut_padded(size);
   CK(c->d_qcnt.ensure(sizeof(unsigned int) * size), what);
   CK(c->d_qkeys.ensure(sizeof(unsigned long long) * padded), what);
   CK(c->d_qcum.ensure(sizeof(long long) * (size + 1)), what);
-  CK(c->d_qbounds.ensure(sizeof(int64_t) * (parts + 1)), what);
   const bool dev_perm = is_device_ptr(perm);
   int32_t *dperm = perm;
   if (!dev_perm) {
@@ -1040,13 +1039,25 @@ static bsvd_status quantile_side(bsvd_ctx *c, const char *what, int64_t size,
   CK(launch_quantile_cut(ids, nnz, size, parts, c->d_qcnt.as<unsigned int>(),
                          c->d_qkeys.as<unsigned long long>(),
                          c->d_qcum.as<long long>(), dperm,
-                         c->d_qbounds.as<int64_t>(), c->d_err.as<int32_t>(),
-                         &c->launches, c->st), what);
+                         dbounds, c->d_err.as<int32_t>(), &c->launches,
+                         c->st), what);
   if (!dev_perm)
     CK(cudaMemcpyAsync(perm, dperm, sizeof(int32_t) * size,
                        cudaMemcpyDeviceToHost, c->st), what);
-  CK(cudaMemcpyAsync(bounds, c->d_qbounds.p, sizeof(int64_t) * (parts + 1),
+  return BSVD_OK;
+}
+
+// Both sides' bounds, one after the other in d_qbounds, to the host: one wait
+// for the device, not one a side.
+static bsvd_status quantile_bounds(bsvd_ctx *c, const char *what, int32_t p,
+                                   int32_t q, int64_t *row_bounds,
+                                   int64_t *col_bounds) {
+  std::vector<int64_t> both((size_t)p + q + 2);
+  CK(cudaMemcpyAsync(both.data(), c->d_qbounds.p, sizeof(int64_t) * both.size(),
                      cudaMemcpyDeviceToHost, c->st), what);
+  CK(cudaStreamSynchronize(c->st), what);
+  std::copy(both.begin(), both.begin() + p + 1, row_bounds);
+  std::copy(both.begin() + p + 1, both.end(), col_bounds);
   return BSVD_OK;
 }
 
@@ -1070,11 +1081,16 @@ bsvd_status bsvd_quantile_grid(bsvd_ctx *c, int64_t m, int64_t n, int64_t nnz,
   CK(cudaMemsetAsync(c->d_err.p, 0, sizeof(int32_t), c->st), "quantile_grid");
   CK(device_view(c, u, sizeof(int32_t) * nnz, c->s_a, &du), "quantile_grid");
   CK(device_view(c, i, sizeof(int32_t) * nnz, c->s_b, &di), "quantile_grid");
+  CK(c->d_qbounds.ensure(sizeof(int64_t) * ((size_t)p + q + 2)),
+     "quantile_grid");
+  int64_t *db = c->d_qbounds.as<int64_t>();
   bsvd_status s = quantile_side(c, "quantile_grid: rows", m, nnz,
-                                (const int32_t *)du, p, row_perm, row_bounds);
+                                (const int32_t *)du, p, row_perm, db);
   if (s != BSVD_OK) return s;
   s = quantile_side(c, "quantile_grid: columns", n, nnz, (const int32_t *)di,
-                    q, col_perm, col_bounds);
+                    q, col_perm, db + p + 1);
+  if (s != BSVD_OK) return s;
+  s = quantile_bounds(c, "quantile_grid", p, q, row_bounds, col_bounds);
   if (s != BSVD_OK) return s;
   return read_errors(c, "quantile_grid");
 }
@@ -1123,14 +1139,17 @@ bsvd_status bsvd_partition_quantile(bsvd_ctx *c, int64_t m, int64_t n,
   // the context); the bounds come to the host for the block layout
   CK(c->d_qperm.ensure(sizeof(int32_t) * m), what);
   CK(c->d_qperm2.ensure(sizeof(int32_t) * n), what);
+  CK(c->d_qbounds.ensure(sizeof(int64_t) * ((size_t)p + q + 2)), what);
+  int64_t *db = c->d_qbounds.as<int64_t>();
   std::vector<int64_t> rb(p + 1), cb(q + 1);
   bsvd_status s = quantile_side(c, "partition_quantile: rows", m, nnz,
                                 (const int32_t *)du, p,
-                                c->d_qperm.as<int32_t>(), rb.data());
+                                c->d_qperm.as<int32_t>(), db);
   if (s == BSVD_OK)
     s = quantile_side(c, "partition_quantile: columns", n, nnz,
                       (const int32_t *)di, q, c->d_qperm2.as<int32_t>(),
-                      cb.data());
+                      db + p + 1);
+  if (s == BSVD_OK) s = quantile_bounds(c, what, p, q, rb.data(), cb.data());
   // the caller's stream takes the upload over in every case, so no later
   // call reuses the staging buffer while it is still being written
   if (forked) CK(cudaStreamWaitEvent(c->st, c->ev_up_join, 0), what);
