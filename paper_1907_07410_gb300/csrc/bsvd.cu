@@ -2245,11 +2245,8 @@ bsvd_status bsvd_sgd_prepare(bsvd_ctx *c, int64_t nnz, const int32_t *u,
   }
   CK(c->d_sgd_hist.ensure(sgd_hist_bytes(nnz)), "sgd_prepare");
   CK(c->d_sgd_start.ensure(ib * (size_t)std::max(c->m, c->n)), "sgd_prepare");
-  // an owner has at most one task in each block of its block row or column
-  const int64_t tmax = std::min<int64_t>(
-      nnz, c->diag ? (o.own_items ? c->n : c->m)
-                   : (o.own_items ? (int64_t)c->p * c->n
-                                  : (int64_t)c->q * c->m));
+  const int64_t tmax = sgd_max_tasks(nnz, c->diag, o.own_items != 0, c->p,
+                                     c->q, c->m, c->n);
   CK(c->d_sgd_first.ensure(ib * (size_t)(tmax + 1)), "sgd_prepare");
   CK(c->d_sgd_ntasks.ensure(sizeof(int64_t)), "sgd_prepare");
   CK(c->d_sgd_u.ensure(sizeof(int32_t) * n1), "sgd_prepare");

@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "sgd_tasks.h"
 
 namespace bsvd {
 
@@ -279,7 +280,7 @@ struct SgdOrder {
   void *key[2], *val[2];     // sort buffers: nnz 8-byte keys, nnz indices
   void *hist;                // sgd_hist_bytes(nnz)
   void *start;               // max(m, n) indices
-  void *task_first;          // written: tasks + 1 indices (room for nnz + 1)
+  void *task_first;          // written: tasks + 1 indices (see sgd_max_tasks)
   int64_t *ntasks;           // written
   int32_t *su, *si;          // written: the ratings in task order
   float *sx;

@@ -72,7 +72,8 @@ __device__ __forceinline__ u64 task_key(const GridDesc &g, const KeyDesc &d,
 // Sort keys. part 0: task key above the minor index; part 1: the minor index
 // alone, part 2: the task key alone of the ratings listed in `list` (two
 // sorts, for grids whose whole key does not fit 64 bits). A rating with an id
-// out of range is reported; its key is that of an existing cell.
+// out of range is reported; its key is that of cell (0, 0) of block 0, whether
+// or not the block has one (sgd_max_tasks counts it).
 template <typename V>
 __global__ void __launch_bounds__(256)
 k_sgd_keys(GridDesc g, KeyDesc d, int64_t nnz, const int32_t *__restrict__ u,
