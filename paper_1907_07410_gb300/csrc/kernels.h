@@ -12,9 +12,10 @@ namespace bsvd {
 // ---- partition (kernels_partition.cu) ----------------------------------
 cudaError_t launch_perm_check(const int32_t *perm, int64_t n, int32_t *seen,
                               int32_t *err, cudaStream_t st);
-// ids[e] += add[b] for e in piece b = [starts[b], starts[b + 1]), b < nb
+// ids[e] += bounds[b] for e in piece b = [starts[b], starts[b + 1]), b < nb;
+// -1 when ids[e] is not below bounds[b + 1] - bounds[b]
 cudaError_t launch_stack_ids(int64_t nnz, int32_t nb, const int64_t *starts,
-                             const int64_t *add, int32_t *ids,
+                             const int64_t *bounds, int32_t *ids,
                              cudaStream_t st);
 cudaError_t launch_count(const GridDesc &g, int64_t nnz, const int32_t *u,
                          const int32_t *i, const float *x, int32_t nblocks,

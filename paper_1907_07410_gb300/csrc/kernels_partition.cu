@@ -32,10 +32,13 @@ constexpr int kRatings = 4;            // ratings a thread has in flight
 constexpr int64_t kChunkedBytes = 256 << 20;
 
 // A batch's ids to the stacked coordinates, in place: 16 bytes of traffic a
-// rating; the piece is found by bisection (the table stays in the L1).
+// rating; the piece is found by bisection (the tables stay in the L1). bounds:
+// where each matrix begins. An id that its matrix does not have becomes -1,
+// which the counting reports: moved along it could be a cell of the next
+// matrix.
 __global__ void k_stack_ids(int64_t nnz, int nb,
                             const int64_t *__restrict__ starts,
-                            const int64_t *__restrict__ add,
+                            const int64_t *__restrict__ bounds,
                             int32_t *__restrict__ ids) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nnz;
        t += (int64_t)gridDim.x * blockDim.x) {
@@ -45,7 +48,9 @@ __global__ void k_stack_ids(int64_t nnz, int nb,
       if (starts[mid] <= t) lo = mid;
       else hi = mid;
     }
-    ids[t] = (int32_t)((uint32_t)ids[t] + (uint32_t)add[lo]);
+    const int32_t id = ids[t];
+    const int64_t first = bounds[lo];
+    ids[t] = id >= 0 && id < bounds[lo + 1] - first ? (int32_t)(first + id) : -1;
   }
 }
 
@@ -705,10 +710,10 @@ cudaError_t launch_count(const GridDesc &g, int64_t nnz, const int32_t *u,
 }
 
 cudaError_t launch_stack_ids(int64_t nnz, int32_t nb, const int64_t *starts,
-                             const int64_t *add, int32_t *ids,
+                             const int64_t *bounds, int32_t *ids,
                              cudaStream_t st) {
   if (nnz <= 0) return cudaSuccess;
-  k_stack_ids<<<grid_for(nnz, 4), 256, 0, st>>>(nnz, nb, starts, add, ids);
+  k_stack_ids<<<grid_for(nnz, 4), 256, 0, st>>>(nnz, nb, starts, bounds, ids);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,40 @@
+"""Ids that one matrix of a batch does not have. Both of a rating's ids out of
+range by the next matrix's offsets make a cell of that matrix in the stacked
+coordinates, so the block diagonal alone does not show them."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_1907_07410_gb300 as bs  # noqa: E402
+
+SIZES = [(8, 8), (9, 5), (6, 7)]
+
+
+def batch(seed=1):
+    rng = np.random.default_rng(seed)
+    us, is_, xs = [], [], []
+    for m, n in SIZES:
+        cells = rng.permutation(m * n)[:20]
+        us.append((cells // n).astype(np.int32))
+        is_.append((cells % n).astype(np.int32))
+        xs.append(rng.integers(1, 6, 20).astype(np.float32))
+    rb, cb = ([0] + list(np.cumsum([s[d] for s in SIZES])) for d in (0, 1))
+    return rb, cb, us, is_, xs
+
+
+@pytest.mark.parametrize("b,u,i", [
+    (0, 8, 8),                  # matrix 1's first cell
+    (1, -1, -1),                # matrix 0's last cell
+    (1, 9 + 5, 5 + 6),          # matrix 2's last cell
+    (2, -17, -13),              # matrix 0's first cell
+    (2, 6, 7), (0, -1, -1),     # outside the batch
+    (0, 2**31 - 1, 2**31 - 1), (2, -2**31, -2**31),
+])
+def test_a_rating_of_another_matrix(b, u, i):
+    rb, cb, us, is_, xs = batch()
+    ctx = bs.Context()
+    us[b][3], is_[b][3] = u, i
+    with pytest.raises(bs.BsvdError):
+        ctx.partition_batch(rb, cb, us, is_, xs)
