@@ -187,8 +187,8 @@ bsvd_status bsvd_partition_diag(bsvd_ctx *ctx, int32_t nb,
  * nu[b] row ids of matrix b in its own coordinates (0 .. m_b - 1), piece b
  * of i and x its columns and ratings (host or device memory, read before the
  * call returns). The pieces are put one after the other on the device, so
- * the caller builds no stacked copy; sum(nu) = sum(ni) = sum(nx). An id that
- * matrix b does not have is an error.
+ * the caller builds no stacked copy. nu[b] = ni[b] = nx[b] for every b. An id
+ * that matrix b does not have is an error.
  */
 bsvd_status bsvd_partition_batch(bsvd_ctx *ctx, int32_t nb,
                                  const int64_t *row_bounds,

@@ -1002,20 +1002,21 @@ bsvd_status bsvd_partition_batch(bsvd_ctx *c, int32_t nb,
     return fail(c, BSVD_EINVAL, "partition_batch: need nb >= 1 and bounds");
   if (!u || !nu || !i || !ni || !x || !nx)
     return fail(c, BSVD_EINVAL, "partition_batch: null piece arrays");
-  int64_t tu = 0, ti = 0, tx = 0;
+  int64_t nnz = 0;
   for (int32_t b = 0; b < nb; ++b) {
     if (nu[b] < 0 || ni[b] < 0 || nx[b] < 0 || (nu[b] && !u[b]) ||
         (ni[b] && !i[b]) || (nx[b] && !x[b]))
       return fail(c, BSVD_EINVAL, "partition_batch: bad pieces of matrix %d", b);
-    tu += nu[b];
-    ti += ni[b];
-    tx += nx[b];
+    // lengths that cancel over the batch would pair one matrix's ids with
+    // another's columns or ratings
+    if (nu[b] != ni[b] || nu[b] != nx[b])
+      return fail(c, BSVD_EINVAL, "partition_batch: matrix %d has %lld rows, "
+                  "%lld columns and %lld ratings", b, (long long)nu[b],
+                  (long long)ni[b], (long long)nx[b]);
+    nnz += nu[b];
   }
-  if (tu != ti || tu != tx)
-    return fail(c, BSVD_EINVAL, "partition_batch: %lld rows, %lld columns and "
-                "%lld ratings", (long long)tu, (long long)ti, (long long)tx);
   const Pieces pieces = {u, nu, i, ni, x, nx};
-  return partition_impl(c, row_bounds[nb], col_bounds[nb], tu, nullptr,
+  return partition_impl(c, row_bounds[nb], col_bounds[nb], nnz, nullptr,
                         nullptr, nullptr, nb, nb, row_bounds, col_bounds,
                         nullptr, nullptr, true, &pieces);
 }

@@ -8,6 +8,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 import paper_1907_07410_gb300 as bs  # noqa: E402
+from paper_1907_07410_gb300 import serve  # noqa: E402
 
 SIZES = [(8, 8), (9, 5), (6, 7)]
 
@@ -38,3 +39,18 @@ def test_a_rating_of_another_matrix(b, u, i):
     us[b][3], is_[b][3] = u, i
     with pytest.raises(bs.BsvdError):
         ctx.partition_batch(rb, cb, us, is_, xs)
+
+
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_lengths_that_cancel_over_the_batch(which):
+    """One array of each kind a matrix, all three of a matrix equally long:
+    here one rating of matrix 0's moves to matrix 1 in one of the three."""
+    rb, cb, us, is_, xs = batch()
+    a = (us, is_, xs)[which]
+    a[0], a[1] = a[0][:-1], np.concatenate([a[0][-1:], a[1]])
+    with pytest.raises((bs.BsvdError, ValueError)):
+        bs.Context().partition_batch(rb, cb, us, is_, xs)
+    reqs = [serve.Request(m, n, 2, u, i, x, u[:1], i[:1])
+            for (m, n), u, i, x in zip(SIZES, us, is_, xs)]
+    with pytest.raises((bs.BsvdError, ValueError)):
+        serve.run_batch(bs.Context(), reqs)
