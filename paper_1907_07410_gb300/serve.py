@@ -226,6 +226,18 @@ class Server:
                 self._done()
 
 
+def _stacked(ids, bounds) -> np.ndarray:
+    """One array of stacked ids from each request's own; -1, which the library
+    reports, in place of an id that its request does not have (moved along it
+    could be a neighbour's)."""
+    a = np.concatenate(ids)
+    lens = [len(p) for p in ids]
+    shape = (len(a),) + (1,) * (a.ndim - 1)
+    first = np.repeat(bounds[:-1], lens).reshape(shape)
+    size = np.repeat(np.diff(bounds), lens).reshape(shape)
+    return np.where((a >= 0) & (a < size), a + first, -1).astype(np.int32)
+
+
 def run_batch(ctx: Context, reqs) -> list:
     """Factorise a batch of requests as one block-diagonal partition and
     return each request's predictions."""
@@ -239,21 +251,21 @@ def run_batch(ctx: Context, reqs) -> list:
         us.append(np.asarray(req.r, np.int32, order="C"))
         is_.append(np.asarray(req.c, np.int32, order="C"))
         xs.append(np.asarray(req.x, np.float32, order="C"))
-        qu.append(np.asarray(req.qr, np.int32) + np.int32(rb[b]))
-        qi.append(np.asarray(req.qc, np.int32) + np.int32(cb[b]))
+        qu.append(np.asarray(req.qr, np.int32))
+        qi.append(np.asarray(req.qc, np.int32))
+        if len(qu[b]) != len(qi[b]):
+            raise ValueError("request %d asks for %d rows and %d columns"
+                             % (b, len(qu[b]), len(qi[b])))
     # the requests' own arrays go to the device, which moves the ids to the
     # stacked coordinates: stacking 16 requests of 6.2 million ratings here
     # took 8 ms of a 12.6 ms batch, and held the interpreter meanwhile
     if all(a.ndim == 1 for a in us + is_ + xs):
         ctx.partition_batch(rb, cb, us, is_, xs)
     else:
-        ctx.partition_diag(
-            rb, cb,
-            np.concatenate([a + np.int32(o) for a, o in zip(us, rb)]),
-            np.concatenate([a + np.int32(o) for a, o in zip(is_, cb)]),
-            np.concatenate(xs))
+        ctx.partition_diag(rb, cb, _stacked(us, rb), _stacked(is_, cb),
+                           np.concatenate(xs))
     ctx.factor([req.k for req in reqs], warn=False)
-    yq = ctx.predict(np.concatenate(qu), np.concatenate(qi))
+    yq = ctx.predict(_stacked(qu, rb), _stacked(qi, cb))
     out, off = [], 0
     for req in reqs:
         nq = len(req.qr)

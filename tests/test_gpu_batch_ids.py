@@ -54,3 +54,48 @@ def test_lengths_that_cancel_over_the_batch(which):
             for (m, n), u, i, x in zip(SIZES, us, is_, xs)]
     with pytest.raises((bs.BsvdError, ValueError)):
         serve.run_batch(bs.Context(), reqs)
+
+
+def requests(b=None, qr=None, qc=None):
+    _, _, us, is_, xs = batch()
+    reqs = [serve.Request(m, n, 2, u, i, x, u[:3], i[:3])
+            for (m, n), u, i, x in zip(SIZES, us, is_, xs)]
+    if b is not None:
+        reqs[b].qr = np.array([0, qr], np.int32)
+        reqs[b].qc = np.array([0, qc], np.int32)
+    return reqs
+
+
+@pytest.mark.parametrize("b,qr,qc", [(0, 8, 8), (1, -1, -1), (1, 14, 11),
+                                     (2, -17, -13), (0, 8, 0), (1, 0, -1)])
+def test_a_prediction_of_another_request(b, qr, qc):
+    """A cell of another request's matrix is no answer to this one's query."""
+    with bs.Context() as ctx:
+        with pytest.raises(bs.BsvdError):
+            serve.run_batch(ctx, requests(b, qr, qc))
+        got = serve.run_batch(ctx, requests())
+    assert [len(y) for y in got] == [3, 3, 3]
+
+
+def test_requests_of_two_dimensions():
+    """Columns of ids are stacked by the host: the same ids, the same checks."""
+    def columns(reqs):
+        for q in reqs:
+            q.r, q.c, q.x = (a.reshape(-1, 1) for a in (q.r, q.c, q.x))
+        return reqs
+    with bs.Context() as ctx:
+        for a, b in zip(serve.run_batch(ctx, columns(requests())),
+                        serve.run_batch(ctx, requests())):
+            assert np.array_equal(a, b)
+        bad = requests()
+        bad[0].r[3], bad[0].c[3] = 8, 8
+        with pytest.raises(bs.BsvdError):
+            serve.run_batch(ctx, columns(bad))
+
+
+def test_queries_whose_lengths_cancel():
+    reqs = requests()
+    reqs[0].qr, reqs[1].qc = reqs[0].qr[:2], reqs[1].qc[:2]
+    with bs.Context() as ctx:
+        with pytest.raises((bs.BsvdError, ValueError)):
+            serve.run_batch(ctx, reqs)
