@@ -306,6 +306,9 @@ struct SgdEpoch {
   SgdRates r;
   int32_t own_items, k;
   int32_t index32 = 0;       // set by launch_sgd_epoch
+  // polls without a task claimed or 32 ratings done anywhere, after which a
+  // wait gives up (kErrTimeout): about half a second
+  unsigned idle_polls = 1u << 21;
   unsigned long long *ctl;
   int32_t *err;
 };

@@ -34,7 +34,7 @@
 // Waiting ends: tasks are claimed in an order in which every task depends
 // only on earlier ones, and a warp works on one task at a time, so the
 // earliest unfinished task never waits for a task that has not been claimed.
-// A wait that sees nothing happen anywhere for kIdlePolls polls (no task
+// A wait that sees nothing happen anywhere for idle_polls polls (no task
 // claimed, no 32 ratings done) gives up: kErrTimeout, and every warp leaves.
 #include <type_traits>
 
@@ -46,7 +46,6 @@ namespace {
 
 typedef unsigned long long u64;
 constexpr unsigned kAll = 0xffffffffu;
-constexpr unsigned kIdlePolls = 1u << 21;   // about half a second of polling
 constexpr unsigned kLookPolls = 1u << 12;   // polls between looks at ctl
 constexpr int kSgdThreads = 256;
 // Resident CTAs per SM: 16 warps. Every warp that waits holds a task, so too
@@ -134,16 +133,20 @@ __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fm
 struct Wait {
   unsigned polls = 0, idle = 0;
   u64 seen = 0;
-  // Called after a poll that failed, by the whole warp; false: give up.
-  __device__ __forceinline__ bool again(volatile u64 *ctl, int32_t *err) {
+  // Called after a poll that failed, by the whole warp; false: give up. The
+  // words are what lane 0 sees of them, so that the whole warp goes on or the
+  // whole warp leaves.
+  __device__ __forceinline__ bool again(const SgdEpoch &a) {
     if (++polls % kLookPolls != 0) return true;
-    if (ctl[2] != 0) return false;
-    const u64 now = ctl[0] + ctl[1];      // both only grow
+    volatile u64 *ctl = a.ctl;
+    if (__shfl_sync(kAll, ctl[2], 0) != 0) return false;
+    // both only grow
+    const u64 now = __shfl_sync(kAll, ctl[0] + ctl[1], 0);
     idle = now == seen ? idle + kLookPolls : 0;
     seen = now;
-    if (idle < kIdlePolls) return true;
+    if (idle < a.idle_polls) return true;
     if ((threadIdx.x & 31) == 0) {
-      atomicOr(err, kErrTimeout);
+      atomicOr(a.err, kErrTimeout);
       ctl[2] = 1;
     }
     return false;
@@ -289,7 +292,7 @@ k_sgd_epoch(SgdEpoch a) {
         bool ok = co[0].is(own_ver);
         if (ALL) ok = ok && co[N - 1].is(own_ver);
         if (__all_sync(kAll, ok)) break;
-        if (!w.again(a.ctl, a.err)) return;
+        if (!w.again(a)) return;
       }
     }
     // PACK: v holds the owner's parameter or the other id's, by lane; else v
@@ -303,7 +306,7 @@ k_sgd_epoch(SgdEpoch a) {
       if (!here(s)) {
         Wait w;
         do {
-          if (!w.again(a.ctl, a.err)) return false;
+          if (!w.again(a)) return false;
           s.cell[0].load(s.row + fo);
           if (ALL) s.cell[N - 1].load(s.row + K * W);
         } while (!here(s));
