@@ -46,6 +46,11 @@ cudaError_t launch_scatter_bf16(const GridDesc &g, const BlockMeta *meta,
                                 const float *mu, __nv_bfloat16 *Wh,
                                 cudaStream_t st);
 
+// Block b's float32 cells (mb x nb, row-major) from the exact Gram's planes.
+cudaError_t launch_rebuild_block(const BlockMeta &bm, int32_t b,
+                                 const __nv_bfloat16 *VX, const float *shift,
+                                 const float *mu, float *out, cudaStream_t st);
+
 // The bf16 planes of a large matrix, every cell of them, chunk by chunk
 // (BlockMeta::ck0). chunks: chunk_words(nchunks) words, the first
 // chunk_slots(nchunks) the ratings per chunk from launch_count (zero before);

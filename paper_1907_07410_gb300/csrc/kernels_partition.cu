@@ -665,6 +665,25 @@ k_fill(const BlockMeta *__restrict__ meta, int32_t nb, int32_t nchunks,
     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
+// One block's cells, row-major, from its planes, as the scatter to the float32
+// arena would have written them.
+__global__ void __launch_bounds__(256)
+k_rebuild_block(BlockMeta bm, int32_t b, const __nv_bfloat16 *__restrict__ VX,
+                const float *__restrict__ shift, const float *__restrict__ mu,
+                float *__restrict__ out) {
+  const float sh = shift[b], mean = mu[b];
+  const __nv_bfloat16 *y = VX + bm.vx_off;
+  const __nv_bfloat16 *mask = y + (int64_t)bm.s128 * bm.L_pad;
+  const int64_t n = (int64_t)bm.mb * bm.nb;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = e / bm.nb, c = e - r * bm.nb;
+    const int64_t cell = bm.trans ? c * bm.L_pad + r : r * bm.L_pad + c;
+    const float x = __fadd_rn(__bfloat162float(y[cell]), sh);
+    out[e] = __bfloat162float(mask[cell]) != 0.f ? __fsub_rn(x, mean) : 0.f;
+  }
+}
+
 int grid_for(int64_t n, int per_thread) {
   int64_t want = (n + 256LL * per_thread - 1) / (256LL * per_thread);
   if (want < 1) want = 1;
@@ -774,6 +793,16 @@ cudaError_t launch_scatter_planes(const GridDesc &g, const BlockMeta *meta,
                                   const float *shift, __nv_bfloat16 *VX,
                                   int32_t *flag, cudaStream_t st) {
   return scatter_to<kToPlanes>(g, meta, nnz, u, i, x, shift, VX, flag, st);
+}
+
+cudaError_t launch_rebuild_block(const BlockMeta &bm, int32_t b,
+                                 const __nv_bfloat16 *VX, const float *shift,
+                                 const float *mu, float *out,
+                                 cudaStream_t st) {
+  const int64_t n = (int64_t)bm.mb * bm.nb;
+  if (n <= 0) return cudaSuccess;
+  k_rebuild_block<<<grid_for(n, 4), 256, 0, st>>>(bm, b, VX, shift, mu, out);
+  return cudaGetLastError();
 }
 
 bool chunked_planes(const GridDesc &g, int64_t nnz, int64_t nchunks,
