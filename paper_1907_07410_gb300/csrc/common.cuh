@@ -215,28 +215,42 @@ __device__ __forceinline__ bool locate(const GridDesc &g, int32_t u,
   return true;
 }
 
-// A CTA's copy of a grid's bounds, for kernels that look up a block per rating
-// or query: at most kTableBounds bounds a side and kTableBlocks blocks (of
-// which the kernels keep what they need beside it). A larger grid is read in
-// place.
+// A CTA's copy of a grid's bounds in shared memory, for kernels that look up a
+// block per rating or query: of the sides that explicit bounds cut (the blocks
+// of the others are found by a division), at most kTableBounds of them.
+// Kernels that keep something of every block beside it do so for at most
+// kTableBlocks blocks. A larger grid is read in place.
 constexpr int kTableBlocks = 512;
-constexpr int kTableBounds = 512;
+constexpr int kTableBounds = 5120;
 
 struct BoundsTable {
-  int32_t rb[kTableBounds + 1], cb[kTableBounds + 1];
-  // Every thread of the CTA; a barrier has to follow.
-  __device__ __forceinline__ void fill(const GridDesc &g) {
-    for (int j = threadIdx.x; j <= g.p; j += blockDim.x)
-      rb[j] = (int32_t)g.row_bounds[j];
-    for (int j = threadIdx.x; j <= g.q; j += blockDim.x)
-      cb[j] = (int32_t)g.col_bounds[j];
+  int32_t *rb = nullptr, *cb = nullptr;
+  // at: bounds_bytes(g) bytes of shared memory. Every thread of the CTA; a
+  // barrier has to follow.
+  __device__ __forceinline__ void fill(const GridDesc &g, void *at) {
+    rb = static_cast<int32_t *>(at);
+    cb = rb + (g.equal_rows ? 0 : g.p + 1);
+    if (!g.equal_rows)
+      for (int j = threadIdx.x; j <= g.p; j += blockDim.x)
+        rb[j] = (int32_t)g.row_bounds[j];
+    if (!g.equal_cols)
+      for (int j = threadIdx.x; j <= g.q; j += blockDim.x)
+        cb[j] = (int32_t)g.col_bounds[j];
   }
 };
+inline int64_t bounds_bytes(const GridDesc &g) {
+  return sizeof(int32_t) * ((g.equal_rows ? 0 : (int64_t)g.p + 1) +
+                            (g.equal_cols ? 0 : (int64_t)g.q + 1));
+}
 inline int32_t grid_blocks(const GridDesc &g) {
   return g.diag ? g.p : g.p * g.q;
 }
+inline bool fits_bounds(const GridDesc &g) {
+  return bounds_bytes(g) <= (int64_t)sizeof(int32_t) * kTableBounds;
+}
+// (at most kTableBlocks blocks have at most 2 kTableBlocks + 2 bounds)
 inline bool fits_table(const GridDesc &g) {
-  return g.p <= kTableBounds && g.q <= kTableBounds &&
+  return g.p <= kTableBlocks && g.q <= kTableBlocks &&
          grid_blocks(g) <= kTableBlocks;
 }
 

@@ -98,7 +98,6 @@ __device__ __forceinline__ long long fixed32(float x) {
 // registers first (16 matrices of the served form: 341 -> 56 us).
 struct CountTable {
   unsigned cnt[kSmemBlocks], lo[kSmemBlocks], hi[kSmemBlocks];
-  BoundsTable bounds;
 };
 
 // Where a cell of a block's bf16 plane is: its chunk and its place in it.
@@ -158,6 +157,8 @@ k_count(GridDesc g, int64_t nnz, const int32_t *__restrict__ u,
         const BlockMeta *__restrict__ meta, unsigned *chunks, uint32_t mask,
         uint2 *__restrict__ where) {
   extern __shared__ unsigned char smem[];
+  // the counts when they fit, CHUNKS: the places (at most kTableBlocks blocks,
+  // so the counts fit), then the bounds
   CountTable &t = *reinterpret_cast<CountTable *>(smem);
   Place *place = reinterpret_cast<Place *>(smem + sizeof(CountTable));
   if (CHUNKS) {
@@ -170,7 +171,11 @@ k_count(GridDesc g, int64_t nnz, const int32_t *__restrict__ u,
     for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
       t.cnt[b] = t.lo[b] = t.hi[b] = 0;
   }
-  if (TABLE) t.bounds.fill(g);
+  BoundsTable bounds;
+  if (TABLE)
+    bounds.fill(g, smem + (CHUNKS ? sizeof(CountTable) +
+                                        sizeof(Place) * kTableBlocks
+                           : use_smem ? sizeof(CountTable) : 0));
   if (threadIdx.x == 0) s_max = 0;
   __syncthreads();
   unsigned int local_max = 0;
@@ -195,7 +200,7 @@ k_count(GridDesc g, int64_t nnz, const int32_t *__restrict__ u,
       bool ok = t0 + k * stride + lane < nnz;
       int32_t blk = -1, ru = 0, ci = 0;
       if (ok) {
-        if (!find_block<TABLE>(g, t.bounds, uu[k], ii[k], &blk, &ru, &ci)) {
+        if (!find_block<TABLE>(g, bounds, uu[k], ii[k], &blk, &ru, &ci)) {
           local_err |= kErrIndex;
           ok = false;
         }
@@ -348,10 +353,13 @@ struct __align__(16) Dest {
 };
 enum { kToFloat, kToBf16, kToPlanes };
 
-struct DestTable {
-  Dest dest[kTableBlocks];
-  BoundsTable bounds;
-};
+// What a CTA keeps in shared memory: nothing, the bounds, or a Dest per block
+// and the bounds. A bisection through bounds in global memory is a chain of
+// loads, which the warp's votes and the rounds of kRatings make longer (900,189
+// ratings on a 30 x 30 quantile grid, counting / float32 scatter: 43 / 22 us
+// with bounds in global memory, 22 / 20 with them here; 36 / 19 a rating at a
+// time).
+enum { kNoTable, kBoundsTable, kFullTable };
 
 template <int TO>
 __device__ __forceinline__ Dest dest_of(const BlockMeta *meta,
@@ -389,19 +397,22 @@ __device__ __forceinline__ int32_t plane_flags(float y, float sub, float lim,
 // number of at most lim, kErrNotHalf when some is not a multiple of one half
 // of at most lim / 2 (four times the sums, in quarters), kErrNotRebuilt when
 // some x is not fl32(y + sub).
-template <int TO, bool TABLE>
+template <int TO, int TABLE>
 __global__ void __launch_bounds__(256)
 k_scatter(GridDesc g, const BlockMeta *__restrict__ meta, int64_t nnz,
           const int32_t *__restrict__ u, const int32_t *__restrict__ it,
           const float *__restrict__ x, const float *__restrict__ sub,
           void *__restrict__ out, int32_t *flag) {
   extern __shared__ __align__(16) unsigned char smem[];
-  DestTable &t = *reinterpret_cast<DestTable *>(smem);
-  if (TABLE) {
-    const int nb = g.diag ? g.p : g.p * g.q;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x)
-      t.dest[b] = dest_of<TO>(meta, sub, b);
-    t.bounds.fill(g);
+  Dest *dest = reinterpret_cast<Dest *>(smem);
+  BoundsTable bounds;
+  if (TABLE != kNoTable) {
+    if (TABLE == kFullTable) {
+      const int nb = g.diag ? g.p : g.p * g.q;
+      for (int b = threadIdx.x; b < nb; b += blockDim.x)
+        dest[b] = dest_of<TO>(meta, sub, b);
+    }
+    bounds.fill(g, smem + (TABLE == kFullTable ? sizeof(Dest) * kTableBlocks : 0));
     __syncthreads();
   }
   int32_t bad = 0;
@@ -422,9 +433,11 @@ k_scatter(GridDesc g, const BlockMeta *__restrict__ meta, int64_t nnz,
     for (int k = 0; k < kRatings; ++k) {
       int32_t blk, ru, ci;
       // ids out of range were flagged when the ratings were counted
-      if (!find_block<TABLE>(g, t.bounds, uu[k], ii[k], &blk, &ru, &ci))
+      if (!find_block<TABLE != kNoTable>(g, bounds, uu[k], ii[k], &blk, &ru,
+                                         &ci))
         continue;
-      const Dest d = TABLE ? t.dest[blk] : dest_of<TO>(meta, sub, blk);
+      const Dest d =
+          TABLE == kFullTable ? dest[blk] : dest_of<TO>(meta, sub, blk);
       if (!(d.flags & 2)) continue;            // another shard's block
       const int32_t r = ru - d.row0, c = ci - d.col0;
       const int64_t cell =
@@ -711,14 +724,15 @@ cudaError_t launch_count(const GridDesc &g, int64_t nnz, const int32_t *u,
   if (nnz <= 0) return cudaSuccess;
   const uint32_t mask = (uint32_t)(chunk_slots(nchunks) - 1);
   // big grids flush many per-CTA histograms: use fewer, longer CTAs
-  int grid = grid_for(nnz, nblocks > 256 ? 16 : 4);
-  const size_t sm = nblocks <= kSmemBlocks ? sizeof(CountTable) : 0;
+  const bool hist = nblocks <= kSmemBlocks;
+  const int grid = grid_for(nnz, hist && nblocks > 256 ? 16 : 4);
+  const size_t sm = hist ? sizeof(CountTable) : 0, bounds = bounds_bytes(g);
   if (chunks)
-    k_count<true, true><<<grid, 256, sm + sizeof(Place) * kTableBlocks, st>>>(
-        g, nnz, u, i, x, nblocks, counts, sums, maxabs_bits, err, meta, chunks,
-        mask, where);
-  else if (fits_table(g))
-    k_count<true, false><<<grid, 256, sm, st>>>(
+    k_count<true, true><<<grid, 256, sm + sizeof(Place) * kTableBlocks + bounds,
+                          st>>>(g, nnz, u, i, x, nblocks, counts, sums,
+                                maxabs_bits, err, meta, chunks, mask, where);
+  else if (fits_bounds(g))
+    k_count<true, false><<<grid, 256, sm + bounds, st>>>(
         g, nnz, u, i, x, nblocks, counts, sums, maxabs_bits, err, meta, chunks,
         mask, where);
   else
@@ -764,11 +778,15 @@ static cudaError_t scatter_to(const GridDesc &g, const BlockMeta *meta,
   if (nnz <= 0) return cudaSuccess;
   const int grid = grid_for(nnz, 4);
   if (fits_table(g))
-    k_scatter<TO, true><<<grid, 256, sizeof(DestTable), st>>>(
+    k_scatter<TO, kFullTable><<<grid, 256,
+                                sizeof(Dest) * kTableBlocks + bounds_bytes(g),
+                                st>>>(g, meta, nnz, u, i, x, sub, out, flag);
+  else if (fits_bounds(g))
+    k_scatter<TO, kBoundsTable><<<grid, 256, bounds_bytes(g), st>>>(
         g, meta, nnz, u, i, x, sub, out, flag);
   else
-    k_scatter<TO, false><<<grid, 256, 0, st>>>(g, meta, nnz, u, i, x, sub, out,
-                                               flag);
+    k_scatter<TO, kNoTable><<<grid, 256, 0, st>>>(g, meta, nnz, u, i, x, sub,
+                                                  out, flag);
   return cudaGetLastError();
 }
 

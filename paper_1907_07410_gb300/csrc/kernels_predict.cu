@@ -32,9 +32,12 @@ struct __align__(16) Place {
 };
 
 struct Table {
-  Place place[kTableBlocks];
+  Place *place = nullptr;        // kTableBlocks of them, then the bounds
   BoundsTable bounds;
 };
+inline size_t table_bytes(const GridDesc &g) {
+  return sizeof(Place) * kTableBlocks + bounds_bytes(g);
+}
 
 __device__ __forceinline__ Place place_of(const PredictArgs &a, int32_t blk) {
   const BlockMeta &bm = a.meta[blk];
@@ -49,10 +52,12 @@ __device__ __forceinline__ Place place_of(const PredictArgs &a, int32_t blk) {
 }
 
 // Every thread of the CTA; ends with a barrier.
-__device__ __forceinline__ void fill_table(const PredictArgs &a, Table &t) {
+__device__ __forceinline__ void fill_table(const PredictArgs &a, Table &t,
+                                           void *smem) {
+  t.place = static_cast<Place *>(smem);
   const int nb = a.g.diag ? a.g.p : a.g.p * a.g.q;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) t.place[b] = place_of(a, b);
-  t.bounds.fill(a.g);
+  t.bounds.fill(a.g, t.place + kTableBlocks);
   __syncthreads();
 }
 
@@ -156,8 +161,8 @@ k_predict(PredictArgs a, int64_t nq, const int32_t *__restrict__ u,
   __shared__ Rows wq[kPredictThreads];
   __shared__ float wdot[kPredictThreads];
   extern __shared__ __align__(16) unsigned char table[];
-  Table &tb = *reinterpret_cast<Table *>(table);
-  if (TABLE) fill_table(a, tb);
+  Table tb;
+  if (TABLE) fill_table(a, tb, table);
   const int w0 = threadIdx.x & ~31, lane = threadIdx.x & 31;
   int32_t bad = 0;
   for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x + w0; t0 < nq;
@@ -235,8 +240,8 @@ k_sqerr(PredictArgs a, int64_t nq, const int32_t *__restrict__ u,
   __shared__ Rows wq[kSqerrThreads];
   __shared__ float wdot[kSqerrThreads];
   extern __shared__ __align__(16) unsigned char table[];
-  Table &tb = *reinterpret_cast<Table *>(table);
-  if (TABLE) fill_table(a, tb);
+  Table tb;
+  if (TABLE) fill_table(a, tb, table);
   const int w0 = threadIdx.x & ~31, lane = threadIdx.x & 31;
   double acc = 0.0;
   long long n = 0;
@@ -336,7 +341,7 @@ cudaError_t launch_predict(const PredictArgs &a, int64_t nq, const int32_t *u,
           a, nq, u, i, yhat, err);
       return cudaGetLastError();
     }
-    k_predict<LPQ, TB><<<grid_for(nq), kPredictThreads, TB ? sizeof(Table) : 0,
+    k_predict<LPQ, TB><<<grid_for(nq), kPredictThreads, TB ? table_bytes(a.g) : 0,
                          st>>>(a, nq, u, i, yhat, err);
     return cudaGetLastError();
   });
@@ -350,7 +355,7 @@ cudaError_t launch_sqerr(const PredictArgs &a, int64_t nq, const int32_t *u,
   const cudaError_t e = by_shape(a, [&](auto l, auto tb) {
     constexpr int LPQ = decltype(l)::value;
     constexpr bool TB = decltype(tb)::value;
-    k_sqerr<LPQ, TB><<<kSqerrBlocks, kSqerrThreads, TB ? sizeof(Table) : 0,
+    k_sqerr<LPQ, TB><<<kSqerrBlocks, kSqerrThreads, TB ? table_bytes(a.g) : 0,
                        st>>>(a, nq, u, i, y, partials, counts, err);
     return cudaGetLastError();
   });
