@@ -325,14 +325,20 @@ k_means(int32_t nblocks, const unsigned long long *counts,
   if ((double)total_c * xmax >= 2147483648.0) {
     if (threadIdx.x == 0) atomicOr(err, kErrSumRange);
   }
+  // An empty block's mean is the mean of all ratings (0 without any). A float64
+  // division is some twenty operations of 63 cycles: where a thread has many
+  // blocks it is taken once (1,350,000 blocks, most of them empty: 4.8 ms with
+  // one for each, 3.7 so; 2,400 blocks: 12.7 us with one for each, 15.2 so).
+  auto mean_of = [](long long sum, unsigned long long count) {
+    return count ? __ddiv_rn(__dmul_rn((double)sum, 0x1p-32), (double)count)
+                 : 0.0;
+  };
+  const bool many = nblocks > 8 * (int)blockDim.x;
+  const double every = many ? mean_of(total_s, total_c) : 0.0;
   for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
     const unsigned long long cb = counts[b];
-    // an empty block's mean is the mean of all ratings (0 without any)
-    const unsigned long long over = cb ? cb : total_c;
-    double m = 0.0;
-    if (over)
-      m = __ddiv_rn(__dmul_rn((double)(cb ? sums[b] : total_s), 0x1p-32),
-                    (double)over);
+    double m = every;
+    if (cb || !many) m = mean_of(cb ? sums[b] : total_s, cb ? cb : total_c);
     mu[b] = __double2float_rn(m);
     if (shift) {
       if (!cb) m = 0.0;

@@ -51,3 +51,21 @@ def test_blocks_of_explicit_bounds(p, q, equal):
                 if prec == bs.BF16:
                     want = torch.from_numpy(np.float32(want)).bfloat16().float()
                 assert np.array_equal(got, np.asarray(want)), b
+
+
+@pytest.mark.parametrize("p,q", [(128, 64), (8193, 1), (91, 91)])
+def test_means_of_many_empty_blocks(p, q):
+    """Around 8,192 blocks, where the mean of all ratings is taken once."""
+    rng = np.random.default_rng(p)
+    m, n = 9000, 100
+    u = rng.integers(0, m, 3000).astype(np.int32)
+    i = ((u * 7 + rng.integers(0, 3, 3000)) % n).astype(np.int32)
+    x = rng.integers(1, 11, 3000).astype(np.float32) / 2
+    part = oracle.partition(m, n, u, i, x, p, q)
+    assert (part.counts == 0).any()
+    for kw in ({}, dict(gram_path=1)):
+        with bs.Context(**kw) as ctx:
+            ctx.partition(m, n, u, i, x, p, q)
+            cnt, mu = ctx.block_stats()
+            assert np.array_equal(cnt, part.counts)
+            assert np.array_equal(mu, part.mu32)
