@@ -79,6 +79,8 @@ __global__ void __launch_bounds__(256)
 k_sgd_keys(GridDesc g, KeyDesc d, int64_t nnz, const int32_t *__restrict__ u,
            const int32_t *__restrict__ it, int part,
            const V *__restrict__ list, u64 *__restrict__ key, int32_t *err) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nnz;
        t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t e = list ? (int64_t)list[t] : t;
@@ -104,6 +106,8 @@ k_sgd_gather(GridDesc g, int64_t nnz, const V *__restrict__ src,
              const float *__restrict__ x, int32_t *__restrict__ su,
              int32_t *__restrict__ si, float *__restrict__ sx,
              V *__restrict__ tile_tasks) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ int starts;
   if (threadIdx.x == 0) starts = 0;
   __syncthreads();
@@ -133,6 +137,8 @@ template <typename V>
 __global__ void __launch_bounds__(1024)
 k_sgd_task_scan(V *__restrict__ tile_tasks, int64_t ntiles,
                 int64_t *__restrict__ ntasks) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ V part[1024];
   V run = 0;
   for (int64_t b = 0; b < ntiles; b += 1024) {
@@ -160,6 +166,8 @@ k_sgd_task_first(int64_t nnz, const u64 *__restrict__ key, int shift,
                  const V *__restrict__ tile_tasks,
                  const int64_t *__restrict__ ntasks,
                  V *__restrict__ task_first) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ int wcount[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t base = (int64_t)blockIdx.x * kRsTile;
@@ -188,6 +196,8 @@ k_sgd_task_first(int64_t nnz, const u64 *__restrict__ key, int shift,
 __global__ void __launch_bounds__(256)
 k_sgd_id_keys(int64_t nnz, const int32_t *__restrict__ id,
               u64 *__restrict__ key) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nnz;
        t += (int64_t)gridDim.x * blockDim.x)
     key[t] = (u64)id[t];
@@ -198,6 +208,8 @@ template <typename V>
 __global__ void __launch_bounds__(256)
 k_sgd_run_start(int64_t nnz, const u64 *__restrict__ key,
                 V *__restrict__ start) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nnz;
        t += (int64_t)gridDim.x * blockDim.x)
     if (t == 0 || key[t] != key[t - 1]) start[key[t]] = (V)t;
@@ -209,6 +221,8 @@ __global__ void __launch_bounds__(256)
 k_sgd_versions(int64_t nnz, const u64 *__restrict__ key,
                const V *__restrict__ pos, const V *__restrict__ start,
                unsigned *__restrict__ ver) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nnz;
        t += (int64_t)gridDim.x * blockDim.x)
     ver[pos[t]] = (unsigned)((V)t - start[key[t]]);
@@ -253,46 +267,59 @@ cudaError_t order_impl(const GridDesc &g, const SgdOrder &o, int64_t nnz,
   const int tbits = bits_of(steps * d.lown * d.slots - 1);
   int cur = 0, shift = d.minor_bits;
   cudaError_t e;
-  if (tbits + d.minor_bits <= 64) {
-    k_sgd_keys<V><<<grid_of(nnz), 256, 0, st>>>(g, d, nnz, u, i, 0, nullptr,
-                                                key[0], err);
+  const dim3 each(grid_of(nnz)), tiles((unsigned)ntiles), cta(256);
+  auto keys = [&](int part, const V *list, u64 *out) -> cudaError_t {
     ++*launches;
+    return launch_pdl(k_sgd_keys<V>, each, cta, 0, st, g, d, nnz, u, i, part,
+                      list, out, err);
+  };
+  if (tbits + d.minor_bits <= 64) {
+    if ((e = keys(0, nullptr, key[0])) != cudaSuccess) return e;
     e = radix_sort<V>(key, val, &cur, true, nnz, tbits + d.minor_bits, hist,
                       total, launches, st);
   } else {
-    k_sgd_keys<V><<<grid_of(nnz), 256, 0, st>>>(g, d, nnz, u, i, 1, nullptr,
-                                                key[0], err);
+    if ((e = keys(1, nullptr, key[0])) != cudaSuccess) return e;
     e = radix_sort<V>(key, val, &cur, true, nnz, d.minor_bits, hist, total,
                       launches, st);
     if (e != cudaSuccess) return e;
-    k_sgd_keys<V><<<grid_of(nnz), 256, 0, st>>>(g, d, nnz, u, i, 2, val[cur],
-                                                key[cur], err);
-    *launches += 2;
+    if ((e = keys(2, val[cur], key[cur])) != cudaSuccess) return e;
     e = radix_sort<V>(key, val, &cur, false, nnz, tbits, hist, total, launches,
                       st);
     shift = 0;
   }
   if (e != cudaSuccess) return e;
-  k_sgd_gather<V><<<(unsigned)ntiles, 256, 0, st>>>(
-      g, nnz, val[cur], key[cur], shift, u, i, x, o.su, o.si, o.sx,
-      tile_tasks);
-  k_sgd_task_scan<V><<<1, 1024, 0, st>>>(tile_tasks, ntiles, o.ntasks);
-  k_sgd_task_first<V><<<(unsigned)ntiles, 256, 0, st>>>(
-      nnz, key[cur], shift, tile_tasks, o.ntasks, first);
+  if ((e = launch_pdl(k_sgd_gather<V>, tiles, cta, 0, st, g, nnz,
+                      (const V *)val[cur], (const u64 *)key[cur], shift, u, i,
+                      x, o.su, o.si, o.sx, tile_tasks)) != cudaSuccess)
+    return e;
+  if ((e = launch_pdl(k_sgd_task_scan<V>, dim3(1), dim3(1024), 0, st,
+                      tile_tasks, ntiles, o.ntasks)) != cudaSuccess)
+    return e;
+  if ((e = launch_pdl(k_sgd_task_first<V>, tiles, cta, 0, st, nnz,
+                      (const u64 *)key[cur], shift, (const V *)tile_tasks,
+                      (const int64_t *)o.ntasks, first)) != cudaSuccess)
+    return e;
   *launches += 3;
   // the versions: other side, then owner
   for (int side = 0; side < 2; ++side) {
     const bool items = (side == 0) != (o.own_items != 0);
     const int32_t *id = items ? o.si : o.su;
     cur = 0;
-    k_sgd_id_keys<<<grid_of(nnz), 256, 0, st>>>(nnz, id, key[0]);
+    if ((e = launch_pdl(k_sgd_id_keys, each, cta, 0, st, nnz, id, key[0])) !=
+        cudaSuccess)
+      return e;
     e = radix_sort<V>(key, val, &cur, true, nnz,
                       bits_of((items ? g.n : g.m) - 1), hist, total, launches,
                       st);
     if (e != cudaSuccess) return e;
-    k_sgd_run_start<V><<<grid_of(nnz), 256, 0, st>>>(nnz, key[cur], start);
-    k_sgd_versions<V><<<grid_of(nnz), 256, 0, st>>>(
-        nnz, key[cur], val[cur], start, side == 0 ? o.other_ver : o.own_ver);
+    if ((e = launch_pdl(k_sgd_run_start<V>, each, cta, 0, st, nnz,
+                        (const u64 *)key[cur], start)) != cudaSuccess)
+      return e;
+    if ((e = launch_pdl(k_sgd_versions<V>, each, cta, 0, st, nnz,
+                        (const u64 *)key[cur], (const V *)val[cur],
+                        (const V *)start,
+                        side == 0 ? o.other_ver : o.own_ver)) != cudaSuccess)
+      return e;
     *launches += 3;
   }
   return cudaGetLastError();
