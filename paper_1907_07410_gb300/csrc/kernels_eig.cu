@@ -54,6 +54,7 @@
 #include <type_traits>
 
 #include "kernels.h"
+#include "quotient.h"
 
 namespace bsvd {
 
@@ -92,18 +93,6 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
   return y;
 }
 constexpr int KC = 32;       // k-chunk of the panel GEMM
-
-// a / b, rounded to nearest, given inv = 1 / b rounded to nearest (Markstein's
-// theorem, "Computation of elementary functions on the IBM RISC System/6000
-// processor", 1990: with the remainder a - b q of a quotient q within one unit
-// in the last place, exact in a fused multiply-add, q + r inv rounds to the
-// nearest). The first correction makes q that close. For operands whose
-// quotient and remainder do not underflow.
-__device__ __forceinline__ float quotient(float a, float b, float inv) {
-  float q = a * inv;
-  q = fmaf(fmaf(-b, q, a), inv, q);
-  return fmaf(fmaf(-b, q, a), inv, q);
-}
 
 __device__ __forceinline__ float hash_uniform(uint64_t seed, uint64_t a,
                                               uint64_t b) {

@@ -4,8 +4,8 @@
 // each rank 512 consecutive keys with a match over equal digits per 32. Up to
 // kRsFewTiles tiles every CTA of the scatter adds up the counts itself, and the
 // scan is left out. The launches overlap (pdl_wait), as the chains that call the
-// sort do: laying out 1,000 / 20,000 / 900,189 ratings for the blocked SGD, 7
-// to 13 passes among 22 to 37 launches, took 139 / 247 / 348 us and takes 82 /
+// sort do: laying out 1,000 / 20,000 / 900,189 ratings for the blocked SGD, 4
+// to 8 passes among 22 to 34 launches, took 139 / 247 / 348 us and takes 82 /
 // 161 / 286.
 #pragma once
 #include "common.cuh"
