@@ -224,18 +224,27 @@ constexpr int kTableBlocks = 512;
 constexpr int kTableBounds = 5120;
 
 struct BoundsTable {
-  int32_t *rb = nullptr, *cb = nullptr;
-  // at: bounds_bytes(g) bytes of shared memory. Every thread of the CTA; a
-  // barrier has to follow.
-  __device__ __forceinline__ void fill(const GridDesc &g, void *at) {
-    rb = static_cast<int32_t *>(at);
-    cb = rb + (g.equal_rows ? 0 : g.p + 1);
+  // Byte offsets in the CTA's dynamic shared memory, not pointers: of a pointer
+  // that a kernel picks at run time the compiler no longer knows the space, and
+  // generic loads took the counting of 90 million ratings from 1.20 to 1.78 ms.
+  uint32_t rb = 0, cb = 0;
+  static __device__ __forceinline__ int32_t *at(uint32_t offset) {
+    extern __shared__ __align__(16) unsigned char bounds_smem[];
+    return reinterpret_cast<int32_t *>(bounds_smem + offset);
+  }
+  __device__ __forceinline__ const int32_t *rows() const { return at(rb); }
+  __device__ __forceinline__ const int32_t *cols() const { return at(cb); }
+  // offset: where bounds_bytes(g) bytes of it are for the table. Every thread
+  // of the CTA; a barrier has to follow.
+  __device__ __forceinline__ void fill(const GridDesc &g, uint32_t offset) {
+    rb = offset;
+    cb = rb + sizeof(int32_t) * (g.equal_rows ? 0 : g.p + 1);
     if (!g.equal_rows)
       for (int j = threadIdx.x; j <= g.p; j += blockDim.x)
-        rb[j] = (int32_t)g.row_bounds[j];
+        at(rb)[j] = (int32_t)g.row_bounds[j];
     if (!g.equal_cols)
       for (int j = threadIdx.x; j <= g.q; j += blockDim.x)
-        cb[j] = (int32_t)g.col_bounds[j];
+        at(cb)[j] = (int32_t)g.col_bounds[j];
   }
 };
 inline int64_t bounds_bytes(const GridDesc &g) {
@@ -266,10 +275,10 @@ __device__ __forceinline__ bool find_block(const GridDesc &g,
   *ci = g.col_perm ? __ldg(g.col_perm + i) : i;
   int32_t bi, bj;
   if (g.equal_rows) bi = (int32_t)((uint32_t)*ru / (uint32_t)g.br);
-  else if (TABLE) bi = upper_index(tb.rb, g.p, *ru);
+  else if (TABLE) bi = upper_index(tb.rows(), g.p, *ru);
   else bi = upper_index(g.row_bounds, g.p, (int64_t)*ru);
   if (g.equal_cols) bj = (int32_t)((uint32_t)*ci / (uint32_t)g.bc);
-  else if (TABLE) bj = upper_index(tb.cb, g.q, *ci);
+  else if (TABLE) bj = upper_index(tb.cols(), g.q, *ci);
   else bj = upper_index(g.col_bounds, g.q, (int64_t)*ci);
   if (g.diag && bi != bj) return false;
   *blk = g.diag ? bi : bi * g.q + bj;

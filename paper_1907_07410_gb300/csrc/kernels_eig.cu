@@ -543,7 +543,9 @@ __device__ int onesided_jacobi(float (*Ac)[P], float (*Vc)[P], int n,
 #pragma unroll
           for (int h = 0; h < RPL; ++h) {
             // which product is rounded first is written out, so that a change
-            // of the code around it changes no result
+            // of the code around it changes no result. At 16 columns the
+            // compiler had chosen the other one in nb; both are as accurate,
+            // and results at k <= 8 stay what they were
             na[h] = fmaf(c, a[h], -__fmul_rn(s, b[h]));
             nb[h] = B == 16 ? fmaf(c, b[h], __fmul_rn(s, a[h]))
                             : fmaf(s, a[h], __fmul_rn(c, b[h]));
@@ -662,7 +664,6 @@ k_rr_solve(const BlockMeta *__restrict__ meta, SolverState *__restrict__ state,
     const int i = e / n, j = e % n;
     const float di = sm.d[i], dj = sm.d[j];
     sm.S[i][j] = (di > 0.f && dj > 0.f) ? sm.S[i][j] / (di * dj) : (i == j ? 0.f : 0.f);
-    sm.Li[i][j] = i == j ? 1.f : 0.f;
   }
   __syncthreads();
   // 3. Cholesky S_n = L L^T, right-looking: for each column j, the pivot

@@ -173,9 +173,8 @@ k_count(GridDesc g, int64_t nnz, const int32_t *__restrict__ u,
   }
   BoundsTable bounds;
   if (TABLE)
-    bounds.fill(g, smem + (CHUNKS ? sizeof(CountTable) +
-                                        sizeof(Place) * kTableBlocks
-                           : use_smem ? sizeof(CountTable) : 0));
+    bounds.fill(g, CHUNKS ? sizeof(CountTable) + sizeof(Place) * kTableBlocks
+                   : use_smem ? sizeof(CountTable) : 0);
   if (threadIdx.x == 0) s_max = 0;
   __syncthreads();
   unsigned int local_max = 0;
@@ -418,7 +417,7 @@ k_scatter(GridDesc g, const BlockMeta *__restrict__ meta, int64_t nnz,
       for (int b = threadIdx.x; b < nb; b += blockDim.x)
         dest[b] = dest_of<TO>(meta, sub, b);
     }
-    bounds.fill(g, smem + (TABLE == kFullTable ? sizeof(Dest) * kTableBlocks : 0));
+    bounds.fill(g, TABLE == kFullTable ? sizeof(Dest) * kTableBlocks : 0);
     __syncthreads();
   }
   int32_t bad = 0;
@@ -703,6 +702,22 @@ k_rebuild_block(BlockMeta bm, int32_t b, const __nv_bfloat16 *__restrict__ VX,
   }
 }
 
+// How much of an SM's 256 KB is shared memory for a kernel, in percent of 228
+// KB; the rest is the L1, which holds what the ratings look up (positions of
+// ids, metadata). Left to itself the runtime makes room for all CTAs that fit.
+// Ten / 90 million ratings on a quantile grid counted with their chunks at 45,
+// 58, 72, 100 %: 152, 146, 168, 209 us / 1.31, 1.16, 1.21, 1.78 ms; the float32
+// scatter with a full table at 45, 58, 100 %: 331, 355, 356 us. The planes'
+// (matrices of a million ratings) 21.1, 20.4, 20.8 us. Without a full table
+// there is little to make room for, and the metadata wants the L1 (900 blocks,
+// five million ratings: 133 us, 253 at 45 %).
+constexpr int kCountCarveout = 58, kScatterCarveout = 45, kPlanesCarveout = 58;
+template <typename K>
+cudaError_t carve_out(K *kernel, int percent) {
+  return cudaFuncSetAttribute(
+      kernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent);
+}
+
 int grid_for(int64_t n, int per_thread) {
   int64_t want = (n + 256LL * per_thread - 1) / (256LL * per_thread);
   if (want < 1) want = 1;
@@ -733,18 +748,15 @@ cudaError_t launch_count(const GridDesc &g, int64_t nnz, const int32_t *u,
   const bool hist = nblocks <= kSmemBlocks;
   const int grid = grid_for(nnz, hist && nblocks > 256 ? 16 : 4);
   const size_t sm = hist ? sizeof(CountTable) : 0, bounds = bounds_bytes(g);
-  if (chunks)
-    k_count<true, true><<<grid, 256, sm + sizeof(Place) * kTableBlocks + bounds,
-                          st>>>(g, nnz, u, i, x, nblocks, counts, sums,
-                                maxabs_bits, err, meta, chunks, mask, where);
-  else if (fits_bounds(g))
-    k_count<true, false><<<grid, 256, sm + bounds, st>>>(
-        g, nnz, u, i, x, nblocks, counts, sums, maxabs_bits, err, meta, chunks,
-        mask, where);
-  else
-    k_count<false, false><<<grid, 256, sm, st>>>(
-        g, nnz, u, i, x, nblocks, counts, sums, maxabs_bits, err, meta, chunks,
-        mask, where);
+  auto kernel = chunks           ? k_count<true, true>
+                : fits_bounds(g) ? k_count<true, false>
+                                 : k_count<false, false>;
+  const size_t bytes = sm + (chunks ? sizeof(Place) * kTableBlocks : 0) +
+                       (chunks || fits_bounds(g) ? bounds : 0);
+  const cudaError_t e = carve_out(kernel, kCountCarveout);
+  if (e != cudaSuccess) return e;
+  kernel<<<grid, 256, bytes, st>>>(g, nnz, u, i, x, nblocks, counts, sums,
+                                   maxabs_bits, err, meta, chunks, mask, where);
   return cudaGetLastError();
 }
 
@@ -783,16 +795,17 @@ static cudaError_t scatter_to(const GridDesc &g, const BlockMeta *meta,
                               int32_t *flag, cudaStream_t st) {
   if (nnz <= 0) return cudaSuccess;
   const int grid = grid_for(nnz, 4);
-  if (fits_table(g))
-    k_scatter<TO, kFullTable><<<grid, 256,
-                                sizeof(Dest) * kTableBlocks + bounds_bytes(g),
-                                st>>>(g, meta, nnz, u, i, x, sub, out, flag);
-  else if (fits_bounds(g))
-    k_scatter<TO, kBoundsTable><<<grid, 256, bounds_bytes(g), st>>>(
-        g, meta, nnz, u, i, x, sub, out, flag);
-  else
-    k_scatter<TO, kNoTable><<<grid, 256, 0, st>>>(g, meta, nnz, u, i, x, sub,
-                                                  out, flag);
+  auto kernel = fits_table(g)    ? k_scatter<TO, kFullTable>
+                : fits_bounds(g) ? k_scatter<TO, kBoundsTable>
+                                 : k_scatter<TO, kNoTable>;
+  const size_t bytes = (fits_table(g) ? sizeof(Dest) * kTableBlocks : 0) +
+                       (fits_bounds(g) ? bounds_bytes(g) : 0);
+  if (fits_table(g)) {
+    const cudaError_t e = carve_out(
+        kernel, TO == kToPlanes ? kPlanesCarveout : kScatterCarveout);
+    if (e != cudaSuccess) return e;
+  }
+  kernel<<<grid, 256, bytes, st>>>(g, meta, nnz, u, i, x, sub, out, flag);
   return cudaGetLastError();
 }
 

@@ -64,7 +64,7 @@ __device__ __forceinline__ void fill_table(const PredictArgs &a, Table &t,
   t.place = static_cast<Place *>(smem);
   const int nb = a.g.diag ? a.g.p : a.g.p * a.g.q;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) t.place[b] = place_of(a, b);
-  t.bounds.fill(a.g, t.place + kTableBlocks);
+  t.bounds.fill(a.g, sizeof(Place) * kTableBlocks);
   __syncthreads();
 }
 
