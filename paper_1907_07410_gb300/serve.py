@@ -227,15 +227,19 @@ class Server:
 
 
 def _stacked(ids, bounds) -> np.ndarray:
-    """One array of stacked ids from each request's own; -1, which the library
-    reports, in place of an id that its request does not have (moved along it
-    could be a neighbour's)."""
+    """One array of stacked ids from each request's own (all of `bounds[0]`'s
+    side, then of the next); -1, which the library reports, in place of an id
+    that its request does not have (moved along it could be a neighbour's)."""
     a = np.concatenate(ids)
     lens = [len(p) for p in ids]
+    first = np.concatenate([b[:-1] for b in bounds]).astype(np.int32)
+    size = np.concatenate([b[1:] - b[:-1] for b in bounds]).astype(np.uint32)
     shape = (len(a),) + (1,) * (a.ndim - 1)
-    first = np.repeat(bounds[:-1], lens).reshape(shape)
-    size = np.repeat(np.diff(bounds), lens).reshape(shape)
-    return np.where((a >= 0) & (a < size), a + first, -1).astype(np.int32)
+    ok = a.view(np.uint32) < np.repeat(size, lens).reshape(shape)
+    a += np.repeat(first, lens).reshape(shape)
+    if not ok.all():
+        a[~ok] = -1
+    return a
 
 
 def run_batch(ctx: Context, reqs) -> list:
@@ -262,10 +266,11 @@ def run_batch(ctx: Context, reqs) -> list:
     if all(a.ndim == 1 for a in us + is_ + xs):
         ctx.partition_batch(rb, cb, us, is_, xs)
     else:
-        ctx.partition_diag(rb, cb, _stacked(us, rb), _stacked(is_, cb),
+        ctx.partition_diag(rb, cb, _stacked(us, [rb]), _stacked(is_, [cb]),
                            np.concatenate(xs))
     ctx.factor([req.k for req in reqs], warn=False)
-    yq = ctx.predict(_stacked(qu, rb), _stacked(qi, cb))
+    q = _stacked(qu + qi, [rb, cb])
+    yq = ctx.predict(q[:len(q) // 2], q[len(q) // 2:])
     out, off = [], 0
     for req in reqs:
         nq = len(req.qr)
