@@ -699,6 +699,7 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
       // exact Gram: planes [Y; M]; bf16 Gram: one bf16 copy of W
       vxoff += (c->cfg.precision == BSVD_BF16 ? 1 : 2) * (int64_t)bm.s128 *
                bm.L_pad;
+      if (c->nblocks > kTableBlocks) continue;   // no chunks (chunked_planes)
       bm.nck = (int32_t)(((int64_t)bm.s128 * bm.L_pad + kPlaneChunk - 1) /
                          kPlaneChunk);
       nchunks += bm.nck;
@@ -851,8 +852,9 @@ static bsvd_status partition_impl(bsvd_ctx *c, int64_t m, int64_t n,
                   c->d_mu.as<float>(),
                   c->tc_planes ? c->d_shift.as<float>() : nullptr,
                   c->tc_planes ? c->d_delta.as<float>() : nullptr,
-                  c->d_err.as<int32_t>(), c->st), "partition: means");
-  c->launches += nnz > 0 ? 2 : 1;
+                  c->d_err.as<int32_t>(), c->st, &c->launches),
+     "partition: means");
+  c->launches += nnz > 0;
   if (c->w32) {
     const bsvd_status ws = write_w();
     if (ws != BSVD_OK) return ws;

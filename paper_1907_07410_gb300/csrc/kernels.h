@@ -28,12 +28,13 @@ cudaError_t launch_count(const GridDesc &g, int64_t nnz, const int32_t *u,
 cudaError_t launch_clear(int32_t nblocks, unsigned long long *counts,
                          long long *sums, unsigned int *maxabs_bits,
                          cudaStream_t st);
-// shift, delta (both or none): the planes' round(mu) and mu - round(mu)
+// shift, delta (both or none): the planes' round(mu) and mu - round(mu).
+// *launches is increased by the number of kernels queued.
 cudaError_t launch_means(int32_t nblocks, const unsigned long long *counts,
                          const long long *sums,
                          const unsigned int *maxabs_bits, float *mu,
                          float *shift, float *delta, int32_t *err,
-                         cudaStream_t st);
+                         cudaStream_t st, int64_t *launches = nullptr);
 // Centred cells into the zeroed float32 arena, or their bf16 rounding into the
 // zeroed bf16 blocks.
 cudaError_t launch_scatter(const GridDesc &g, const BlockMeta *meta,
