@@ -2225,6 +2225,7 @@ bsvd_status bsvd_sgd_prepare(bsvd_ctx *c, int64_t nnz, const int32_t *u,
   if (!c->parted) return fail(c, BSVD_ESTATE, "sgd_prepare: no partition");
   if (nnz < 0 || nnz >= ((int64_t)1 << 40) || (nnz > 0 && (!u || !i || !x)))
     return fail(c, BSVD_EINVAL, "sgd_prepare: bad arguments");
+  // the interface's limit; the order itself would take any width (two sorts)
   for (int32_t j = 0; j < c->q; ++j)
     if (c->cb[j + 1] - c->cb[j] >= ((int64_t)1 << 23))
       return fail(c, BSVD_EINVAL, "sgd_prepare: a block is too wide");

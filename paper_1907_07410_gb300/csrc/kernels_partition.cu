@@ -13,8 +13,8 @@
 // what it needs of each block in shared memory (BoundsTable, Dest); from
 // global memory a rating's six or more lookups touch up to 32 lines per warp
 // each. A thread takes kRatings ratings at a time, so that their loads
-// overlap: counting 90 million ratings into 256 blocks takes 0.90 ms (1.43
-// before both). A random access of the L2 a rating (the position of an id, a
+// overlap: counting 90 million ratings into 256 blocks took 0.90 ms with both
+// (1.43 before). A random access of the L2 a rating (the position of an id, a
 // counter, a list's place) takes about 75 us per ten million, which is what
 // the counting and listing of a large matrix are bound by.
 #include <type_traits>
@@ -488,12 +488,12 @@ k_scatter(GridDesc g, const BlockMeta *__restrict__ meta, int64_t nnz,
 // planes cost a 32-byte DRAM sector each, written part by part at 25 to 30
 // billion a second whatever the order of issue: 10.8 million ratings in
 // 3.8 GB of planes took 635 us after a memset of 590. Instead the ratings are
-// counted by chunk of 2^14 cells (in k_count), put into their chunk's list
-// (k_bucket, 4 bytes each: 14 bits of place, the bf16 offset), and a CTA lays
+// counted by chunk of 2^13 cells (in k_count), put into their chunk's list
+// (k_bucket, 4 bytes each: 13 bits of place, the bf16 offset), and a CTA lays
 // out one chunk at a time in shared memory and stores it as it is (k_fill),
-// zeros included: 157 + 667 us and 60 more in k_count; 17 GB of one plane and
-// 90 million ratings 1.5 + 3.0 ms and 0.3, from 2.7 + 3.8; 0.35 GB and 6.2
-// million in a batch 116 + 71 and 42 us, from 348 + 60. Chunks of 2^12 or 2^14
+// zeros included: 158 + 673 us and 52 more in k_count; 17 GB of one plane and
+// 90 million ratings 1.56 + 3.10 ms, from 2.7 + 3.8; 0.35 GB and 6.2 million in
+// a batch 118 + 71 us, from 348 + 60. Chunks of 2^12 or 2^14
 // cells are within 5 % on the large ones; 2^14 costs the batch 60 us (fewer
 // counters, more waiting at each).
 //
@@ -611,7 +611,8 @@ k_bucket(int nb, const BlockMeta *__restrict__ meta, int64_t nnz,
 
 // out: every cell of the planes (PLANES = 2: the offsets, then the mask).
 // The chunk in shared memory is zero between chunks: the cells that were set
-// are set back. Three CTAs an SM, so that two work while one's store drains.
+// are set back. Six CTAs an SM with two planes, eleven with one (as many chunks
+// fit its shared memory), so that the others work while one's store drains.
 constexpr int kFillThreads = kPlaneChunk / 64;
 constexpr int kHold = 4;
 template <int PLANES>
