@@ -401,19 +401,20 @@ static cudaError_t few(const PredictArgs &a, int64_t nq, const int32_t *u,
 // than two thirds of a wave (kFewLanes of 152 x 2,048), one lane a sum. Beyond
 // that two lanes for rows of up to five chunks, one for rows of one or two, up
 // to kFewQueries, and then, or for longer rows at once, the form with a table
-// (for grids without one the same, with the blocks read in place; rows of
-// three chunks stay with two lanes there). Short rows leave that form's lanes
-// idle: without the rule ten million queries at kp = 4 took 143 us. The kernel
-// alone, us, a lane per query / now: 4 x 4 equal blocks, 40,000 queries kp = 8
-// 3.4 / 3.1, 20 4.4 / 3.6, 40 6.0 / 3.9; 120,000 queries 4.4 / 4.5, 6.4 / 5.9,
-// 9.7 / 7.1; ten million kp = 4 107 / 91, 8 137 / 123, 12 175 / 150, 20 260 /
-// 205, 40 491 / 281, 56 685 / 307; 900 blocks, ten million kp = 8 184 / 180, 20
-// 310 / 254, 56 751 / 423.
+// (for grids without one the same, with the blocks read in place; with explicit
+// bounds, rows of three chunks stay with two lanes there). Short rows leave that
+// form's lanes idle: without the rule ten million queries at kp = 4 took 143 us.
+// The kernel alone, us, a lane per query / now: 4 x 4 equal blocks, 40,000
+// queries kp = 8 3.4 / 3.1, 20 4.4 / 3.6, 40 6.0 / 3.9; 120,000 queries 4.4 /
+// 4.5, 6.4 / 5.9, 9.7 / 7.1; ten million kp = 4 107 / 91, 8 137 / 123, 12 175 /
+// 150, 20 260 / 205, 40 491 / 281, 56 685 / 307; 900 blocks, ten million kp = 8
+// 184 / 180, 12 224 / 202, 20 310 / 254, 56 751 / 423.
 cudaError_t launch_predict(const PredictArgs &a, int64_t nq, const int32_t *u,
                            const int32_t *i, float *yhat, int32_t *err,
                            cudaStream_t st) {
   if (nq <= 0) return cudaSuccess;
   const int n4 = a.kp / 4;
+  const bool equal = a.g.equal_rows && a.g.equal_cols;
   return by_shape(a, [&](auto l, auto tb) {
     constexpr int LPQ = decltype(l)::value;
     constexpr bool TB = decltype(tb)::value;
@@ -427,7 +428,7 @@ cudaError_t launch_predict(const PredictArgs &a, int64_t nq, const int32_t *u,
     } else {
       if (LPQ == 2 && nq * 2 > kFewLanes && (nq <= 2 * kFewQueries || !TB))
         return few<LPQ, 1>(a, nq, u, i, yhat, err, st);
-      if (n4 <= 5 && (nq <= kFewQueries || (n4 == 3 && !TB)))
+      if (n4 <= 5 && (nq <= kFewQueries || (n4 == 3 && !TB && !equal)))
         return few<LPQ, 2>(a, nq, u, i, yhat, err, st);
       k_predict<LPQ, TB><<<grid_for(nq), kPredictThreads,
                            TB ? table_bytes(a.g) : 0, st>>>(a, nq, u, i, yhat,
